@@ -156,11 +156,8 @@ ibl_status ibl_destroy(ibl_ctx* c) {
   if (c->d_status) cudaFree(c->d_status);
   if (c->d_mass_parts) cudaFree(c->d_mass_parts);
   if (c->d_mass_ref) cudaFree(c->d_mass_ref);
-  if (c->d_pt_perm) cudaFree(c->d_pt_perm);
-  if (c->d_pt_bins) cudaFree(c->d_pt_bins);
-  if (c->d_pt_mom) cudaFree(c->d_pt_mom);
-  if (c->d_pt_sbase) cudaFree(c->d_pt_sbase);
-  if (c->d_pt_swts) cudaFree(c->d_pt_swts);
+  for (void* p : {c->d_pt_slot, c->d_pt_rec, c->d_pt_wts, c->d_pt_vd, c->d_pt_off, c->d_pt_mom})
+    if (p) cudaFree(p);
   for (auto& ev : c->stage_ev)
     if (ev) cudaEventDestroy(ev);
   for (auto& ev : c->prof_ev) cudaEventDestroy(ev);

@@ -92,13 +92,14 @@ struct ibl_ctx {
   double* d_mass_ref = nullptr;    // [0] total at initialisation, [1] last total, [2] checks
   int mass_every = 500;            // steps between mass checks (0: off)
   double mass_tol = 0.0;           // relative drift bound (0: default for the precision)
-  int* d_pt_perm = nullptr;      // point operators: sorted point order (pt_cap ints)
-  int* d_pt_bins = nullptr;      // point operators: per-tile counters / offsets (n_tiles ints)
+  // point operators (points.cu), grown on demand
+  void* d_pt_slot = nullptr;      // bin and rank of each point (pt_cap points)
+  void* d_pt_rec = nullptr;       // first stencil nodes and index, in bin order
+  void* d_pt_wts = nullptr;       // double-float delta weights, in bin order
+  void* d_pt_vd = nullptr;        // V ds as double-floats, in bin order
   size_t pt_cap = 0;
-  void* d_pt_mom = nullptr;       // point operators: drho and u* of every cell (4 N values)
-  void* d_pt_sbase = nullptr;     // point operators: stencil bases (3 per point)
-  void* d_pt_swts = nullptr;      // point operators: double-float stencil weights (12 per point)
-  size_t pt_st_cap = 0;
+  void* d_pt_off = nullptr;       // per bin: counters, offsets, heavy marks
+  void* d_pt_mom = nullptr;       // drho and u* of every cell (4 N values)
   size_t pt_mom_bytes = 0;
   int sticky = 0;                // host copy of status bits seen so far
   std::string err;

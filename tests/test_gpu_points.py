@@ -200,3 +200,65 @@ def test_points_full_size_sampled(ibl):
         w = oib.phi(r[0]) * oib.phi(r[1]) * oib.phi(r[2])
         want[c] = (w[:, None] * V).sum(axis=0)
     assert np.abs(got - want).max() < 1e-11
+
+
+# Grids whose axes end in a tile of one or two nodes, fit one tile, or have an
+# odd width; the last row packs enough points around one tile (over 16384) for
+# the path that such tiles take.
+TILE_EDGES = [
+    (19, (8, 9, 17), [W.PERIODIC] * 6, 500, 1.0),
+    (19, (10, 18, 34), [W.PERIODIC] * 6, 500, 1.0),
+    (19, (17, 8, 33), [W.PERIODIC, W.PERIODIC, W.BOUNCEBACK, W.BOUNCEBACK, W.PERIODIC, W.PERIODIC], 500, 1.0),
+    (9, (1, 34, 65), [W.PERIODIC, W.PERIODIC, W.BOUNCEBACK, W.BOUNCEBACK, 0, 0], 500, 1.0),
+    (9, (1, 33, 8), [W.PERIODIC] * 6, 500, 1.0),
+    (19, (24, 24, 40), [W.PERIODIC] * 6, 20000, 0.2),
+]
+
+
+@pytest.mark.parametrize("q,shape,bc,m,span", TILE_EDGES)
+def test_spread_points_tile_edges(ibl, q, shape, bc, m, span):
+    """Each term is rounded to 2^-46 in two parts (2 quanta), and its weight and
+    products carry a few 2^-47 of its size (under 8e-15): a cell that n terms
+    reach is off by at most n (2 quanta + 8e-15 max|V ds|), the one large value
+    apart."""
+    ctx, sim = _pair(ibl, q, "fp32", shape, bc, 0)
+    d = sim.lat.d
+    periodic = [bc[2 * a] == W.PERIODIC for a in range(3)]
+    X = _cloud(m, shape, periodic, seed=31)
+    if span < 1.0:
+        X = 6.0 + span * X
+    rng = np.random.default_rng(5)
+    V = rng.uniform(-0.05, 0.05, size=(m, d))
+    V[0] = 300.0   # above the range of the short conversion
+    ds = rng.uniform(0.5, 1.5, size=m)
+    n = shape[0] * shape[1] * shape[2]
+    whole = torch.empty(d * n + 1, dtype=torch.float64, device="cuda")
+    out = whole[1:].view((d,) + shape)   # 8-byte aligned only
+    ctx.ibl_spread_points(_dev(X), _dev(V), _dev(ds), out)
+    Dm = oib.spread_matrix(X[:, :d], shape, sim.periodic)
+    ref = oib.spread(Dm, V, ds, shape)
+    terms = oib.spread(abs(Dm) > 0, np.ones((m, d)), np.ones(m), shape)
+    err = np.abs(out.cpu().numpy() - ref)
+    size = np.abs(V * ds[:, None]).max(axis=1)
+    first = oib.spread(abs(Dm) > 0, (np.arange(m) == 0)[:, None] * np.ones((m, d)), np.ones(m), shape)
+    bound = terms * (2 * FIX_QUANTUM + 8e-15 * size[1:].max()) + first * 8e-15 * size[0]
+    assert (err <= bound).all()
+    assert torch.equal(out, ctx.ibl_spread_points(_dev(X), _dev(V), _dev(ds)))
+
+
+@pytest.mark.parametrize("q,prec,shape,bc", CASES[:3])
+def test_interpolate_binned_order(ibl, q, prec, shape, bc):
+    """Clouds between an eighth of the grid's nodes and all of them are binned
+    before they pull at every node: the same bits as a few points at a time."""
+    ctx, sim = _pair(ibl, q, prec, shape, bc, 2)
+    periodic = [bc[2 * a] == W.PERIODIC for a in range(3)]
+    nodes = 64 if q == 19 else 16
+    n = shape[0] * shape[1] * shape[2]
+    m = n // nodes - 1
+    assert n // 8 <= m * nodes < n
+    X = _cloud(m, shape, periodic, seed=41)
+    U, rho = ctx.ibl_interpolate_points(_dev(X))
+    part = max(1, n // (9 * nodes))
+    parts = [ctx.ibl_interpolate_points(_dev(X[k:k + part])) for k in range(0, m, part)]
+    assert torch.equal(U, torch.cat([p[0] for p in parts]))
+    assert torch.equal(rho, torch.cat([p[1] for p in parts]))
