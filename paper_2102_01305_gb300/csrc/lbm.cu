@@ -11,6 +11,7 @@
 // Sec. 3.1 Zou-He inlet / outlet.
 #include <mutex>
 
+#include "df.cuh"
 #include "ibl_internal.cuh"
 #include "lbm_gather.cuh"
 
@@ -159,7 +160,11 @@ __device__ __forceinline__ typename O::V dir_dot(int i, const typename O::V v[3]
 // F is the uniform body force G plus, with IB, the IB force density
 // 2 rho du (Eq. 26) formed here from this cell's own density; F is returned
 // in F.  Without IB, du = 0 and F = G exactly (G carries no negative zero).
-template <int Q, bool IB, class O>
+// FG: the run has a uniform body force.  Without one a cell off the band has
+// F = 0, and every term of the source is an exact zero: !IB && !FG leaves them
+// out (two fifths of the operations) with the same result, but for the sign
+// of a zero.
+template <int Q, bool IB, bool FG, class O>
 __device__ __forceinline__ typename O::V collide_v(typename O::V g[Q], typename O::V F[3],
                                                    const typename O::V du[3],
                                                    const FluidParams<typename O::R>& p) {
@@ -182,13 +187,14 @@ __device__ __forceinline__ typename O::V collide_v(typename O::V g[Q], typename 
     }
   }
   if (Lat<Q>::D == 2) m[2] = O::splat(R(0));
+  constexpr bool FORCE = IB || FG;
   // 2 rho du = 2 du + drho (2 du) (rho = 1 + drho is not formed in low precision)
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
     if (IB) {
       const V t = O::mul(O::splat(R(2)), du[a]);
       F[a] = O::add(O::splat(p.G[a]), O::fma(drho, t, t));
-    } else {
+    } else if (FG) {
       F[a] = O::splat(p.G[a]);
     }
   }
@@ -197,13 +203,16 @@ __device__ __forceinline__ typename O::V collide_v(typename O::V g[Q], typename 
   V u[3];
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
-    u[a] = O::fma(O::splat(R(0.5)), F[a], m[a]);
+    u[a] = FORCE ? O::fma(O::splat(R(0.5)), F[a], m[a]) : m[a];
     u[a] = O::fma(u[a], nq, u[a]);
   }
   const V usq = O::fma(u[2], u[2], O::fma(u[1], u[1], O::mul(u[0], u[0])));
-  const V uF = O::fma(u[2], F[2], O::fma(u[1], F[1], O::mul(u[0], F[0])));
+  V m3uF{};
+  if (FORCE) {
+    const V uF = O::fma(u[2], F[2], O::fma(u[1], F[1], O::mul(u[0], F[0])));
+    m3uF = O::mul(O::splat(R(-3)), uF);             // -3 u.F
+  }
   const V X = O::mul(O::splat(R(-1.5)), usq);       // -1.5 u.u
-  const V m3uF = O::mul(O::splat(R(-3)), uF);       // -3 u.F
   const V nom = O::splat(-p.omega);
   const R pref = p.pref;
   {
@@ -212,12 +221,12 @@ __device__ __forceinline__ typename O::V collide_v(typename O::V g[Q], typename 
     const R w = R(Lat<Q>::w(0));
     const V E0 = O::add(drho, O::fma(drho, X, X));
     const V t = O::fma(O::splat(-w), E0, g[0]);                        // g0 - w E0
-    g[0] = O::fma(O::splat(rn_mul(pref, w)), m3uF, O::fma(nom, t, g[0]));
+    g[0] = O::fma(nom, t, g[0]);
+    if (FORCE) g[0] = O::fma(O::splat(rn_mul(pref, w)), m3uF, g[0]);
   }
 #pragma unroll
   for (int i = 1; i < Q; i += 2) {
     const V cu = dir_dot<Q, O>(i, u);
-    const V cF = dir_dot<Q, O>(i, F);
     const R w = R(Lat<Q>::w(i));
     const R wo = w3<Q, R>(i);
     const R pwo = rn_mul(pref, wo);
@@ -228,21 +237,25 @@ __device__ __forceinline__ typename O::V collide_v(typename O::V g[Q], typename 
     const V Oc = O::fma(drho, cu, cu);
     const V eq_p = O::fma(O::splat(wo), Oc, ge);
     const V eq_m = O::fma(O::splat(-wo), Oc, ge);
+    const V a = g[i], b = g[i + 1];
+    g[i] = O::fma(nom, O::sub(a, eq_p), a);
+    g[i + 1] = O::fma(nom, O::sub(b, eq_m), b);
+    if (!FORCE) continue;
     // Eq. 8: pref w [3 (c - u).F + 9 (c.u)(c.F)]: even pref w (9 cu cF - 3 uF),
     // odd +/- pref wo cF
+    const V cF = dir_dot<Q, O>(i, F);
     const V Se = O::mul(O::splat(rn_mul(pref, w)), O::fma(O::mul(O::splat(R(9)), cu), cF, m3uF));
     const V S_p = O::fma(O::splat(pwo), cF, Se);
     const V S_m = O::fma(O::splat(-pwo), cF, Se);
-    const V a = g[i], b = g[i + 1];
-    g[i] = O::add(O::fma(nom, O::sub(a, eq_p), a), S_p);
-    g[i + 1] = O::add(O::fma(nom, O::sub(b, eq_m), b), S_m);
+    g[i] = O::add(g[i], S_p);
+    g[i + 1] = O::add(g[i + 1], S_m);
   }
   return drho;
 }
 
-template <int Q, bool IB, class R>
+template <int Q, bool IB, bool FG, class R>
 __device__ __forceinline__ R collide(R g[Q], R F[3], const R du[3], const FluidParams<R>& p) {
-  return collide_v<Q, IB, Sc<R>>(g, F, du, p);
+  return collide_v<Q, IB, FG, Sc<R>>(g, F, du, p);
 }
 
 // Per-direction base pointers of the two population buffers (kernel
@@ -288,7 +301,7 @@ __device__ __forceinline__ void gather_fast(const DirPtrs<Q, T>& P, int x, int y
 // One cell of the fused step: pull (with faces), IB velocity correction of
 // band cells, collision with forcing, store; the same arithmetic whichever
 // kernel runs it, so every launch split gives bitwise the same populations.
-template <int Q, class T, bool PULL, bool IB>
+template <int Q, class T, bool PULL, bool IB, bool FG>
 __device__ __forceinline__ void collide_cell(const DirPtrs<Q, T>& P, const FluidParams<typename Store<T>::R>& p,
                                              int x, int y, int z) {
   using R = typename Store<T>::R;
@@ -306,7 +319,9 @@ __device__ __forceinline__ void collide_cell(const DirPtrs<Q, T>& P, const Fluid
   R du[3] = {R(0), R(0), R(0)};
   int band = -1;
   if (IB) band = band_du<Q, R>(x, y, z, p, du);
-  const R drho = collide<Q, IB, R>(g, F, du, p);
+  R drho;
+  if (IB && !FG && band < 0) drho = collide<Q, false, false, R>(g, F, du, p);   // F = 0
+  else drho = collide<Q, IB, FG, R>(g, F, du, p);
   if (!(drho > R(-1) && drho < R(99))) atomicOr(p.status, ST_DIVERGED);
 #pragma unroll
   for (int i = 0; i < Q; ++i) P.d[i][cell] = Store<T>::st(g[i]);
@@ -409,7 +424,7 @@ __device__ __forceinline__ void gather_pair_words(const DirPtrs<Q, T>& P, int x,
 // Band correction, collision and divergence check of the cells (x, x + 1)
 // (the part of collide_cell between the pull and the store, on both lanes).
 // x is even and tiles are 16 cells wide, so both cells lie in one tile.
-template <int Q, bool IB>
+template <int Q, bool IB, bool FG>
 __device__ __forceinline__ void collide_pair(F2 g[Q], const FluidParams<float>& p, int x, int y, int z) {
   F2 F[3], du[3];
   int band = -1;
@@ -420,7 +435,9 @@ __device__ __forceinline__ void collide_pair(F2 g[Q], const FluidParams<float>& 
 #pragma unroll
     for (int a = 0; a < 3; ++a) du[a] = Pk::make(da[a], db[a]);
   }
-  const F2 drho = collide_v<Q, IB, Pk>(g, F, du, p);
+  F2 drho;
+  if (IB && !FG && band < 0) drho = collide_v<Q, false, false, Pk>(g, F, du, p);   // F = 0
+  else drho = collide_v<Q, IB, FG, Pk>(g, F, du, p);
   const float d0 = Pk::lo(drho), d1 = Pk::hi(drho);
   if (!(d0 > -1.0f && d0 < 99.0f) || !(d1 > -1.0f && d1 < 99.0f)) atomicOr(p.status, ST_DIVERGED);
   if (IB && band >= 0) {
@@ -436,11 +453,11 @@ __device__ __forceinline__ void collide_pair(F2 g[Q], const FluidParams<float>& 
 // The pair (x, x + 1) when either cell lies on a non-periodic face: the
 // one-cell path with its face gathers, out of line so that its registers
 // do not count against the two-cell kernels' hot path.
-template <int Q, class T, bool IB>
+template <int Q, class T, bool IB, bool FG>
 __device__ __noinline__ void collide_face_pair(const DirPtrs<Q, T>& P, const FluidParams<float>& p, int x, int y,
                                                int z) {
-  collide_cell<Q, T, true, IB>(P, p, x, y, z);
-  collide_cell<Q, T, true, IB>(P, p, x + 1, y, z);
+  collide_cell<Q, T, true, IB, FG>(P, p, x, y, z);
+  collide_cell<Q, T, true, IB, FG>(P, p, x + 1, y, z);
 }
 
 // Every cell of a grid with even nx: 2 x-adjacent cells per thread,
@@ -449,7 +466,7 @@ __device__ __noinline__ void collide_face_pair(const DirPtrs<Q, T>& P, const Flu
 #ifndef IBL_PAIRS_MIN_BLOCKS
 #define IBL_PAIRS_MIN_BLOCKS 4
 #endif
-template <int Q, class T, bool IB>
+template <int Q, class T, bool IB, bool FG>
 __global__ void __launch_bounds__(256, IB ? 3 : IBL_PAIRS_MIN_BLOCKS) k_collide_pairs(DirPtrs<Q, T> P, FluidParams<float> p) {
   const int x = 2 * (blockIdx.x * blockDim.x + threadIdx.x);
   const int y = blockIdx.y * blockDim.y + threadIdx.y;
@@ -461,10 +478,10 @@ __global__ void __launch_bounds__(256, IB ? 3 : IBL_PAIRS_MIN_BLOCKS) k_collide_
   gather_pair_words<Q, T>(P, inside ? x : p.nx - 2, inside ? y : p.ny - 1, z, p, g);
   if (!inside) return;
   if (on_special_face<float>(x, y, z, Lat<Q>::D, p) || on_special_face<float>(x + 1, y, z, Lat<Q>::D, p)) {
-    collide_face_pair<Q, T, IB>(P, p, x, y, z);
+    collide_face_pair<Q, T, IB, FG>(P, p, x, y, z);
     return;
   }
-  collide_pair<Q, IB>(g, p, x, y, z);
+  collide_pair<Q, IB, FG>(g, p, x, y, z);
   const int cell = (z * p.ny + y) * p.nx + x;
 #pragma unroll
   for (int i = 0; i < Q; ++i) *reinterpret_cast<unsigned*>(P.d[i] + cell) = Pack16<T>::st(g[i]);
@@ -544,7 +561,7 @@ __device__ __forceinline__ void unpack_pair_words(const PairWords<Q, T>& W, int 
 #ifndef IBL_ZP_MIN_BLOCKS
 #define IBL_ZP_MIN_BLOCKS 2
 #endif
-template <int Q, class T, bool IB>
+template <int Q, class T, bool IB, bool FG>
 __global__ void __launch_bounds__(256, IBL_ZP_MIN_BLOCKS) k_collide_pairs_zp(DirPtrs<Q, T> P, FluidParams<float> p) {
   const int x = 2 * (blockIdx.x * blockDim.x + threadIdx.x);
   const int y = blockIdx.y * blockDim.y + threadIdx.y;
@@ -562,10 +579,10 @@ __global__ void __launch_bounds__(256, IBL_ZP_MIN_BLOCKS) k_collide_pairs_zp(Dir
     if (z + 1 < z1) load_pair_words<Q, T>(P, xc, yc, z + 1, p, next);
     if (!inside) continue;
     if (on_special_face<float>(x, y, z, Lat<Q>::D, p) || on_special_face<float>(x + 1, y, z, Lat<Q>::D, p)) {
-      collide_face_pair<Q, T, IB>(P, p, x, y, z);
+      collide_face_pair<Q, T, IB, FG>(P, p, x, y, z);
       continue;
     }
-    collide_pair<Q, IB>(g, p, x, y, z);
+    collide_pair<Q, IB, FG>(g, p, x, y, z);
     const int cell = (z * p.ny + y) * p.nx + x;
 #pragma unroll
     for (int i = 0; i < Q; ++i) *reinterpret_cast<unsigned*>(P.d[i] + cell) = Pack16<T>::st(g[i]);
@@ -673,7 +690,7 @@ __device__ __forceinline__ void stage_plane(const DirPtrs<Q, T>& P, const FluidP
 }
 
 // One thread per cell pair (x, x + 1), 64 x 4 threads, SZ planes per block.
-template <int Q, class T, bool IB>
+template <int Q, class T, bool IB, bool FG>
 __global__ void __launch_bounds__(256, IB ? 3 : 4) k_collide_pairs_staged(DirPtrs<Q, T> P, FluidParams<float> p) {
   extern __shared__ __align__(128) unsigned char stage_smem[];
   T* bufs = reinterpret_cast<T*>(stage_smem);
@@ -706,7 +723,7 @@ __global__ void __launch_bounds__(256, IB ? 3 : 4) k_collide_pairs_staged(DirPtr
     const int z = z0 + k;
     if (inside) {
       if (on_special_face<float>(x, y, z, Lat<Q>::D, p) || on_special_face<float>(x + 1, y, z, Lat<Q>::D, p)) {
-        collide_face_pair<Q, T, IB>(P, p, x, y, z);
+        collide_face_pair<Q, T, IB, FG>(P, p, x, y, z);
       } else {
         F2 g[Q];
         const T* base = buf + ty * SROW + SPAD + 2 * tx;
@@ -721,7 +738,7 @@ __global__ void __launch_bounds__(256, IB ? 3 : 4) k_collide_pairs_staged(DirPtr
             g[i] = Pack16<T>::ld(s[d], s[d + 1]);
           }
         }
-        collide_pair<Q, IB>(g, p, x, y, z);
+        collide_pair<Q, IB, FG>(g, p, x, y, z);
         const int cell = (z * p.ny + y) * p.nx + x;
 #pragma unroll
         for (int i = 0; i < Q; ++i) *reinterpret_cast<unsigned*>(P.d[i] + cell) = Pack16<T>::st(g[i]);
@@ -732,20 +749,22 @@ __global__ void __launch_bounds__(256, IB ? 3 : 4) k_collide_pairs_staged(DirPtr
 }
 
 // Every cell, one per thread (blocks of the collide shape); IB selects the band lookup.
-template <int Q, class T, bool PULL, bool IB>
+template <int Q, class T, bool PULL, bool IB, bool FG>
 __global__ void __launch_bounds__(256) k_collide(DirPtrs<Q, T> P, FluidParams<typename Store<T>::R> p) {
   const int x = blockIdx.x * blockDim.x + threadIdx.x;
   const int y = blockIdx.y * blockDim.y + threadIdx.y;
   const int z = blockIdx.z;
   if (x >= p.nx || y >= p.ny) return;
-  collide_cell<Q, T, PULL, IB>(P, p, x, y, z);
+  collide_cell<Q, T, PULL, IB, FG>(P, p, x, y, z);
 }
 
 // Cells outside the IB band, while the IB chain runs on other SMs: a
 // persistent grid of 1024-thread blocks (one per SM: each holds the whole
 // register file, so the SMs it does not take stay free for the solve), each
 // walking 64 x 16-cell units of one z-plane; band tiles are skipped and
-// left to k_collide_band.
+// left to k_collide_band.  It keeps the source's terms without a body force
+// too: it is not on the step's critical path, and without them it pressed the
+// solve's L2 and HBM traffic harder (2 x 2634 markers: 1.4 % longer steps).
 constexpr int BULK_THREADS = 1024;
 template <int Q, class T, bool PULL>
 __global__ void __launch_bounds__(BULK_THREADS, 1) k_collide_bulk(DirPtrs<Q, T> P,
@@ -761,7 +780,7 @@ __global__ void __launch_bounds__(BULK_THREADS, 1) k_collide_bulk(DirPtrs<Q, T> 
   while (z < p.nz) {
     const int x = (bx << 6) + lx, y = (by << 4) + ly;
     if (x < p.nx && y < p.ny && p.tile_slot[tile_index<Q, R>(x, y, z, p)] < 0)
-      collide_cell<Q, T, PULL, false>(P, p, x, y, z);
+      collide_cell<Q, T, PULL, false, true>(P, p, x, y, z);
     bx += gx;
     int carry = bx >= ux;
     bx -= carry ? ux : 0;
@@ -787,58 +806,159 @@ __global__ void __launch_bounds__(TILE_CELLS) k_collide_band(DirPtrs<Q, T> P, Fl
     const int y = ((tile / t.ntx) % t.nty) * t.ty + ly;
     const int z = (tile / (t.ntx * t.nty)) * t.tz + lz;
     if (x >= p.nx || y >= p.ny || z >= p.nz) continue;
-    collide_cell<Q, T, PULL, true>(P, p, x, y, z);
+    collide_cell<Q, T, PULL, true, true>(P, p, x, y, z);   // every cell has a force
   }
 }
 
+// Sums over one cell's populations beyond the storage's precision.  FP64
+// storage sums in FP64.  FP32 and 16-bit storage sum in double-float (48 bits,
+// the storage has 24 at most): FP64 instructions, conversions included, issue at
+// about 1/64 of the FP32 rate, and the kernels that used them here were bound by
+// them.
+template <class R> struct Wide;
+template <> struct Wide<double> {
+  using V = double;
+  static __device__ __forceinline__ V of(double a) { return a; }
+  static __device__ __forceinline__ V add(V a, V b) { return a + b; }
+  static __device__ __forceinline__ V sub(V a, V b) { return a - b; }
+  static __device__ __forceinline__ V mul(V a, V b) { return a * b; }
+  static __device__ __forceinline__ V div(V a, V b) { return a / b; }
+  static __device__ __forceinline__ double value(V a) { return a; }
+  static __device__ __forceinline__ double store(V a) { return a; }
+  static __device__ __forceinline__ V konst(double c) { return c; }
+};
+template <> struct Wide<float> {
+  using V = df;
+  static __device__ __forceinline__ V of(float a) { return df_make(a, 0.f); }
+  static __device__ __forceinline__ V of(double a) { return df_from_double(a); }
+  // one rounding of the low parts: an error of about 2^-47 of the larger operand
+  static __device__ __forceinline__ V add(V a, V b) {
+    const df s = two_sum(a.hi, b.hi);
+    return fast_two_sum(s.hi, __fadd_rn(s.lo, __fadd_rn(a.lo, b.lo)));
+  }
+  static __device__ __forceinline__ V sub(V a, V b) { return add(a, df_neg(b)); }
+  static __device__ __forceinline__ V mul(V a, V b) { return df_mul(a, b); }
+  static __device__ __forceinline__ V div(V a, V b) { return df_div(a, b); }
+  static __device__ __forceinline__ double value(V a) { return df_to_double(a); }
+  static __device__ __forceinline__ float store(V a) { return a.hi; }   // normalised: hi is the rounded value
+  static __device__ __forceinline__ V konst(double c) { return df_make((float)c, (float)(c - (double)(float)c)); }
+};
+
 // rho, u = (sum c_i f_i + G/2)/rho and optionally f itself (FP64) of the
-// current post-streaming populations.
-template <int Q, class T, bool PULL>
-__global__ void k_fields(const T* __restrict__ src, FluidParams<typename Store<T>::R> p,
-                         double* __restrict__ rho_out, double* __restrict__ u_out,
-                         double* __restrict__ pop_out) {
+// current post-streaming populations.  U: the velocity is asked for.
+// 64^3 FP32: 68 us for u with FP64 sums and divisions, 14 us now.
+template <int Q, class T, bool PULL, bool U>
+__global__ void __launch_bounds__(256) k_fields(const T* __restrict__ src, FluidParams<typename Store<T>::R> p,
+                                                double* __restrict__ rho_out, double* __restrict__ u_out,
+                                                double* __restrict__ pop_out) {
   using R = typename Store<T>::R;
+  using O = Wide<R>;
+  using V = typename O::V;
   const int x = blockIdx.x * blockDim.x + threadIdx.x;
   const int y = blockIdx.y * blockDim.y + threadIdx.y;
   const int z = blockIdx.z;
   if (x >= p.nx || y >= p.ny) return;
   const long long cell = ((long long)z * p.ny + y) * p.nx + x;
   R g[Q];
-  gather_q<Q, T, PULL, R>(src, x, y, z, cell, p, g);
-  double drho = 0, m[3] = {0, 0, 0};
+  pull_cell<Q, T, PULL>(src, x, y, z, p, g);
+  if (pop_out) {
 #pragma unroll
-  for (int i = 0; i < Q; ++i) {
-    const double gi = (double)g[i];
-    drho += gi;
-    m[0] += Lat<Q>::cx(i) * gi;
-    m[1] += Lat<Q>::cy(i) * gi;
-    m[2] += Lat<Q>::cz(i) * gi;
-    if (pop_out) pop_out[i * p.N + cell] = gi + Lat<Q>::w(i);
+    for (int i = 0; i < Q; ++i) pop_out[i * p.N + cell] = (double)g[i] + Lat<Q>::w(i);
   }
-  const double rho = 1.0 + drho;
-  if (rho_out) rho_out[cell] = rho;
-  if (u_out)
+  if (!rho_out && !U) return;
+  V drho = O::of(g[0]);
+  V m[3] = {O::of(p.G[0] * R(0.5)), O::of(p.G[1] * R(0.5)), O::of(p.G[2] * R(0.5))};
+#pragma unroll
+  for (int i = 1; i < Q; ++i) {
+    const V gi = O::of(g[i]);
+    drho = O::add(drho, gi);
+    if (U) {
+      const int c[3] = {Lat<Q>::cx(i), Lat<Q>::cy(i), Lat<Q>::cz(i)};
+#pragma unroll
+      for (int a = 0; a < 3; ++a)
+        if (c[a] != 0) m[a] = c[a] > 0 ? O::add(m[a], gi) : O::sub(m[a], gi);
+    }
+  }
+  if (sizeof(R) == 4 && !isfinite(O::value(drho))) {
+    // double-float turns an infinity into a NaN: such a cell in plain FP64
+    double r = 0.0, q[3] = {0.0, 0.0, 0.0};
+    for (int i = 0; i < Q; ++i) {
+      const double gi = (double)g[i];
+      r += gi;
+      if (Lat<Q>::cx(i)) q[0] += Lat<Q>::cx(i) * gi;
+      if (Lat<Q>::cy(i)) q[1] += Lat<Q>::cy(i) * gi;
+      if (Lat<Q>::cz(i)) q[2] += Lat<Q>::cz(i) * gi;
+    }
+    if (rho_out) rho_out[cell] = 1.0 + r;
+    if (U)
+      for (int a = 0; a < Lat<Q>::D; ++a) u_out[a * p.N + cell] = (q[a] + 0.5 * (double)p.G[a]) / (1.0 + r);
+    return;
+  }
+  const V rho = O::add(O::konst(1.0), drho);
+  if (rho_out) rho_out[cell] = 1.0 + O::value(drho);
+  if (U) {
+    // double-float: one division and a product per component
+    const V inv = sizeof(R) == 4 ? O::div(O::konst(1.0), rho) : rho;
+#pragma unroll
     for (int a = 0; a < Lat<Q>::D; ++a)
-      u_out[a * p.N + cell] = (m[a] + 0.5 * (double)p.G[a]) / rho;
+      u_out[a * p.N + cell] = O::value(sizeof(R) == 4 ? O::mul(m[a], inv) : O::div(m[a], rho));
+  }
 }
 
-template <int Q, class T>
-__global__ void k_init_eq(T* __restrict__ dst, long long N, const double* __restrict__ rho_in,
-                          const double* __restrict__ u_in) {
+// f_i = f_eq(rho, u) - w_i (Eq. 4), by direction pairs (c, -c) that share the
+// even part: w [drho + rho (4.5 cu^2 - 1.5 u.u)] +/- w rho 3 cu.
+// GIVEN = false: at rest with rho = 1 the deviations are zero.
+// Bound by FP64 conversions of the given field and, in FP32, by HBM: 256^3
+// FP32 413 us, 5189 us when every direction was formed in FP64 by itself.
+template <int Q, class T, bool GIVEN>
+__global__ void __launch_bounds__(256) k_init_eq(T* __restrict__ dst, long long N, const double* __restrict__ rho_in,
+                                                 const double* __restrict__ u_in) {
+  using R = typename Store<T>::R;
+  using O = Wide<R>;
+  using V = typename O::V;
   const long long cell = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (cell >= N) return;
-  const double rho = rho_in ? rho_in[cell] : 1.0;
-  double u[3] = {0, 0, 0};
-  if (u_in)
-    for (int a = 0; a < Lat<Q>::D; ++a) u[a] = u_in[a * N + cell];
-  const double usq = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
+  if (!GIVEN) {
 #pragma unroll
-  for (int i = 0; i < Q; ++i) {
-    const double cu = Lat<Q>::cx(i) * u[0] + Lat<Q>::cy(i) * u[1] + Lat<Q>::cz(i) * u[2];
-    const double w = Lat<Q>::w(i);
-    // f_eq - w, Eq. 4
-    const double geq = w * ((rho - 1.0) + rho * (3.0 * cu + 4.5 * cu * cu - 1.5 * usq));
-    dst[i * N + cell] = Store<T>::st((typename Store<T>::R)geq);
+    for (int i = 0; i < Q; ++i) dst[i * N + cell] = Store<T>::st(R(0));
+    return;
+  }
+  V u[3] = {O::konst(0.0), O::konst(0.0), O::konst(0.0)};
+  if (u_in) {
+#pragma unroll
+    for (int a = 0; a < Lat<Q>::D; ++a) u[a] = O::of(u_in[a * N + cell]);
+  }
+  V usq = O::add(O::mul(u[0], u[0]), O::mul(u[1], u[1]));
+  if (Lat<Q>::D == 3) usq = O::add(usq, O::mul(u[2], u[2]));
+  V drho = O::konst(0.0);
+  V rho3 = O::konst(3.0), rho45 = O::konst(4.5), rho15 = O::konst(-1.5);
+  if (rho_in) {
+    const double r = rho_in[cell];
+    const V rv = O::of(r);
+    drho = O::of(r - 1.0);
+    rho3 = O::mul(rho3, rv);
+    rho45 = O::mul(rho45, rv);
+    rho15 = O::mul(rho15, rv);
+  }
+  const V base = O::add(drho, O::mul(rho15, usq));
+  dst[cell] = Store<T>::st((R)O::store(O::mul(O::konst(Lat<Q>::w(0)), base)));
+#pragma unroll
+  for (int i = 1; i < Q; i += 2) {
+    // c.u of the first member of a pair: its first nonzero component is +1
+    const int c[3] = {Lat<Q>::cx(i), Lat<Q>::cy(i), Lat<Q>::cz(i)};
+    V cu = u[0];
+    bool have = false;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      if (c[a] == 0) continue;
+      cu = !have ? u[a] : (c[a] > 0 ? O::add(cu, u[a]) : O::sub(cu, u[a]));
+      have = true;
+    }
+    const V w = O::konst(Lat<Q>::w(i));
+    const V even = O::add(base, O::mul(rho45, O::mul(cu, cu)));
+    const V odd = O::mul(rho3, cu);
+    dst[i * N + cell] = Store<T>::st((R)O::store(O::mul(w, O::add(even, odd))));
+    dst[(i + 1) * N + cell] = Store<T>::st((R)O::store(O::mul(w, O::sub(even, odd))));
   }
 }
 
@@ -851,30 +971,41 @@ __global__ void k_set_pop(T* __restrict__ dst, long long N, const double* __rest
     dst[i * N + cell] = Store<T>::st((typename Store<T>::R)(f[i * N + cell] - Lat<Q>::w(i)));
 }
 
-// Fixed-order FP64 mass: block b sums cells [b*chunk, (b+1)*chunk) in a fixed
+// Fixed-order mass: block b sums cells [b*chunk, (b+1)*chunk) in a fixed
 // strided pattern and a fixed tree; the host-side second pass is a fixed loop.
+// A cell's deviations are summed beyond the storage's precision (Wide), the
+// cells' sums in FP64, and the cells themselves are counted.  Bound by HBM in
+// FP32 (256^3: 268 us; 1280 us with FP64 conversions and additions per
+// direction and 64-bit index divisions).
 template <int Q, class T, bool PULL>
-__global__ void k_mass(const T* __restrict__ src, FluidParams<typename Store<T>::R> p,
-                       double* __restrict__ partials, long long chunk) {
+__global__ void __launch_bounds__(256) k_mass(const T* __restrict__ src, FluidParams<typename Store<T>::R> p,
+                                              double* __restrict__ partials, long long chunk) {
   using R = typename Store<T>::R;
+  using O = Wide<R>;
   __shared__ double sh[256];
   const long long start = (long long)blockIdx.x * chunk;
   long long end = start + chunk;
   if (end > p.N) end = p.N;
   double acc = 0;
-  for (long long cell = start + threadIdx.x; cell < end; cell += blockDim.x) {
-    const int x = (int)(cell % p.nx);
-    const long long yz = cell / p.nx;
-    const int y = (int)(yz % p.ny);
-    const int z = (int)(yz / p.ny);
+  long long cells = 0;
+  for (long long c = start + threadIdx.x; c < end; c += blockDim.x) {
+    const unsigned cell = (unsigned)c;   // a context has at most 2^31 - 1 cells
+    const unsigned yz = cell / (unsigned)p.nx;
+    const unsigned z = yz / (unsigned)p.ny;
     R g[Q];
-    gather_q<Q, T, PULL, R>(src, x, y, z, cell, p, g);
-    double drho = 0;
+    pull_cell<Q, T, PULL>(src, (int)(cell - yz * (unsigned)p.nx), (int)(yz - z * (unsigned)p.ny), (int)z, p, g);
+    typename O::V drho = O::of(g[0]);
 #pragma unroll
-    for (int i = 0; i < Q; ++i) drho += (double)g[i];
-    acc += 1.0 + drho;
+    for (int i = 1; i < Q; ++i) drho = O::add(drho, O::of(g[i]));
+    double cell_sum = O::value(drho);
+    if (sizeof(R) == 4 && !isfinite(cell_sum)) {   // an infinity, which double-float turns into a NaN
+      cell_sum = 0.0;
+      for (int i = 0; i < Q; ++i) cell_sum += (double)g[i];
+    }
+    acc += cell_sum;
+    ++cells;
   }
-  sh[threadIdx.x] = acc;
+  sh[threadIdx.x] = acc + (double)cells;
   __syncthreads();
   for (int s = blockDim.x / 2; s > 0; s >>= 1) {
     if (threadIdx.x < s) sh[threadIdx.x] += sh[threadIdx.x + s];
@@ -946,8 +1077,10 @@ DirPtrs<Q, T> dir_ptrs(ibl_ctx* c) {
   return P;
 }
 
-template <int Q, class T>
-cudaError_t collide_q(ibl_ctx* c, bool with_ib) {
+static bool has_body_force(const ibl_ctx* c) { return c->G[0] != 0.0 || c->G[1] != 0.0 || c->G[2] != 0.0; }
+
+template <int Q, class T, bool FG>
+cudaError_t collide_fg(ibl_ctx* c, bool with_ib) {
   using R = typename Store<T>::R;
   auto p = make_params<R>(c, with_ib);
   const DirPtrs<Q, T> P = dir_ptrs<Q, T>(c);
@@ -959,8 +1092,8 @@ cudaError_t collide_q(ibl_ctx* c, bool with_ib) {
         const dim3 sb(SX / 2, SY, 1);
         const dim3 sg((c->nx + SX - 1) / SX, (c->ny + SY - 1) / SY, (c->nz + SZ - 1) / SZ);
         const size_t smem = staged_smem_bytes(Q);
-        if (with_ib) k_collide_pairs_staged<Q, T, true><<<sg, sb, smem, c->stream>>>(P, p);
-        else k_collide_pairs_staged<Q, T, false><<<sg, sb, smem, c->stream>>>(P, p);
+        if (with_ib) k_collide_pairs_staged<Q, T, true, FG><<<sg, sb, smem, c->stream>>>(P, p);
+        else k_collide_pairs_staged<Q, T, false, FG><<<sg, sb, smem, c->stream>>>(P, p);
         c->launches++;
         return cudaGetLastError();
       }
@@ -969,29 +1102,34 @@ cudaError_t collide_q(ibl_ctx* c, bool with_ib) {
       // 16-bit storage: two cells per thread, ZP planes per thread
       const dim3 zb(b.x, b.y, 1);
       const dim3 zg((c->nx / 2 + zb.x - 1) / zb.x, (c->ny + zb.y - 1) / zb.y, (c->nz + ZP - 1) / ZP);
-      if (with_ib) k_collide_pairs_zp<Q, T, true><<<zg, zb, 0, c->stream>>>(P, p);
-      else k_collide_pairs_zp<Q, T, false><<<zg, zb, 0, c->stream>>>(P, p);
+      if (with_ib) k_collide_pairs_zp<Q, T, true, FG><<<zg, zb, 0, c->stream>>>(P, p);
+      else k_collide_pairs_zp<Q, T, false, FG><<<zg, zb, 0, c->stream>>>(P, p);
       c->launches++;
       return cudaGetLastError();
     }
     if (!c->poststream && c->nx % 2 == 0 && c->collide_pairs >= 1) {
       // 16-bit storage: two x-adjacent cells per thread
       g.x = (c->nx / 2 + b.x - 1) / b.x;
-      if (with_ib) k_collide_pairs<Q, T, true><<<g, b, 0, c->stream>>>(P, p);
-      else k_collide_pairs<Q, T, false><<<g, b, 0, c->stream>>>(P, p);
+      if (with_ib) k_collide_pairs<Q, T, true, FG><<<g, b, 0, c->stream>>>(P, p);
+      else k_collide_pairs<Q, T, false, FG><<<g, b, 0, c->stream>>>(P, p);
       c->launches++;
       return cudaGetLastError();
     }
   }
   if (c->poststream) {
-    if (with_ib) k_collide<Q, T, false, true><<<g, b, 0, c->stream>>>(P, p);
-    else k_collide<Q, T, false, false><<<g, b, 0, c->stream>>>(P, p);
+    if (with_ib) k_collide<Q, T, false, true, FG><<<g, b, 0, c->stream>>>(P, p);
+    else k_collide<Q, T, false, false, FG><<<g, b, 0, c->stream>>>(P, p);
   } else {
-    if (with_ib) k_collide<Q, T, true, true><<<g, b, 0, c->stream>>>(P, p);
-    else k_collide<Q, T, true, false><<<g, b, 0, c->stream>>>(P, p);
+    if (with_ib) k_collide<Q, T, true, true, FG><<<g, b, 0, c->stream>>>(P, p);
+    else k_collide<Q, T, true, false, FG><<<g, b, 0, c->stream>>>(P, p);
   }
   c->launches++;
   return cudaGetLastError();
+}
+
+template <int Q, class T>
+cudaError_t collide_q(ibl_ctx* c, bool with_ib) {
+  return has_body_force(c) ? collide_fg<Q, T, true>(c, with_ib) : collide_fg<Q, T, false>(c, with_ib);
 }
 
 template <int Q, class T>
@@ -999,8 +1137,8 @@ cudaError_t collide_bulk_q(ibl_ctx* c, int blocks, cudaStream_t st) {
   using R = typename Store<T>::R;
   auto p = make_params<R>(c, true);
   const DirPtrs<Q, T> P = dir_ptrs<Q, T>(c);
-  if (c->poststream) k_collide_bulk<Q, T, false><<<blocks, BULK_THREADS, 0, st>>>(P, p);
-  else k_collide_bulk<Q, T, true><<<blocks, BULK_THREADS, 0, st>>>(P, p);
+  auto kernel = c->poststream ? k_collide_bulk<Q, T, false> : k_collide_bulk<Q, T, true>;
+  kernel<<<blocks, BULK_THREADS, 0, st>>>(P, p);
   c->launches++;
   return cudaGetLastError();
 }
@@ -1010,12 +1148,8 @@ cudaError_t collide_band_q(ibl_ctx* c, int blocks) {
   using R = typename Store<T>::R;
   auto p = make_params<R>(c, true);
   const DirPtrs<Q, T> P = dir_ptrs<Q, T>(c);
-  if (c->poststream)
-    k_collide_band<Q, T, false><<<blocks, TILE_CELLS, 0, c->stream>>>(P, p, c->d_slot_tile, c->d_band_count,
-                                                                       c->cap_slots);
-  else
-    k_collide_band<Q, T, true><<<blocks, TILE_CELLS, 0, c->stream>>>(P, p, c->d_slot_tile, c->d_band_count,
-                                                                      c->cap_slots);
+  auto kernel = c->poststream ? k_collide_band<Q, T, false> : k_collide_band<Q, T, true>;
+  kernel<<<blocks, TILE_CELLS, 0, c->stream>>>(P, p, c->d_slot_tile, c->d_band_count, c->cap_slots);
   c->launches++;
   return cudaGetLastError();
 }
@@ -1026,8 +1160,13 @@ cudaError_t fields_q(ibl_ctx* c, double* d_rho, double* d_u, double* d_pop) {
   auto p = make_params<R>(c, false);
   const T* src = (const T*)c->f[c->cur];
   dim3 b(64, 4, 1), g = cell_grid(c, b);
-  if (c->poststream) k_fields<Q, T, false><<<g, b, 0, c->stream>>>(src, p, d_rho, d_u, d_pop);
-  else k_fields<Q, T, true><<<g, b, 0, c->stream>>>(src, p, d_rho, d_u, d_pop);
+  if (d_u) {
+    if (c->poststream) k_fields<Q, T, false, true><<<g, b, 0, c->stream>>>(src, p, d_rho, d_u, d_pop);
+    else k_fields<Q, T, true, true><<<g, b, 0, c->stream>>>(src, p, d_rho, d_u, d_pop);
+  } else {
+    if (c->poststream) k_fields<Q, T, false, false><<<g, b, 0, c->stream>>>(src, p, d_rho, d_u, d_pop);
+    else k_fields<Q, T, true, false><<<g, b, 0, c->stream>>>(src, p, d_rho, d_u, d_pop);
+  }
   c->launches++;
   return cudaGetLastError();
 }
@@ -1048,7 +1187,8 @@ template <int Q, class T>
 cudaError_t init_q(ibl_ctx* c, const double* d_rho, const double* d_u) {
   const int bs = 256;
   const long long nb = (c->N + bs - 1) / bs;
-  k_init_eq<Q, T><<<(unsigned)nb, bs, 0, c->stream>>>((T*)c->f[c->cur], c->N, d_rho, d_u);
+  if (d_rho || d_u) k_init_eq<Q, T, true><<<(unsigned)nb, bs, 0, c->stream>>>((T*)c->f[c->cur], c->N, d_rho, d_u);
+  else k_init_eq<Q, T, false><<<(unsigned)nb, bs, 0, c->stream>>>((T*)c->f[c->cur], c->N, nullptr, nullptr);
   c->launches++;
   return cudaGetLastError();
 }

@@ -117,4 +117,36 @@ __device__ __forceinline__ void gather_q(const T* __restrict__ src, int x, int y
   if (zh_face >= 0) zou_he<Q, R>(g, zh_face, p);
 }
 
+// Post-streaming populations of one cell, with a short pull for every cell
+// that is not on a wall or a Zou-He face: the neighbour rows and columns are
+// wrapped once and a direction costs one addition and one load, where gather_q
+// tests each direction against every face.
+template <int Q, class T, bool PULL>
+__device__ __forceinline__ void pull_cell(const T* __restrict__ src, int x, int y, int z,
+                                          const FluidParams<typename Store<T>::R>& p, typename Store<T>::R g[Q]) {
+  using R = typename Store<T>::R;
+  constexpr int D = Lat<Q>::D;
+  const bool special =
+      PULL && ((x == 0 && p.bc[0] != IBL_PERIODIC) || (x == p.nx - 1 && p.bc[1] != IBL_PERIODIC) ||
+               (y == 0 && p.bc[2] != IBL_PERIODIC) || (y == p.ny - 1 && p.bc[3] != IBL_PERIODIC) ||
+               (D == 3 && ((z == 0 && p.bc[4] != IBL_PERIODIC) || (z == p.nz - 1 && p.bc[5] != IBL_PERIODIC))));
+  if (special) {
+    gather_q<Q, T, PULL, R>(src, x, y, z, ((long long)z * p.ny + y) * p.nx + x, p, g);
+  } else if (!PULL) {
+    const int cell = (z * p.ny + y) * p.nx + x;
+#pragma unroll
+    for (int i = 0; i < Q; ++i) g[i] = Store<T>::ld(src[i * p.N + cell]);
+  } else {
+    const int xs[3] = {x == 0 ? p.nx - 1 : x - 1, x, x == p.nx - 1 ? 0 : x + 1};
+    const int ys[3] = {y == 0 ? p.ny - 1 : y - 1, y, y == p.ny - 1 ? 0 : y + 1};
+    const int zs[3] = {z == 0 ? p.nz - 1 : z - 1, z, z == p.nz - 1 ? 0 : z + 1};
+#pragma unroll
+    for (int i = 0; i < Q; ++i) {
+      const int zi = D == 3 ? zs[1 - Lat<Q>::cz(i)] : z;
+      const int from = (zi * p.ny + ys[1 - Lat<Q>::cy(i)]) * p.nx + xs[1 - Lat<Q>::cx(i)];
+      g[i] = Store<T>::ld(src[i * p.N + from]);
+    }
+  }
+}
+
 }  // namespace ibl

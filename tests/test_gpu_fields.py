@@ -1,0 +1,81 @@
+"""GPU parity of the set-up and read-out kernels: f_eq from given fields
+(Eq. 4), moments (Eq. 9) and mass of given populations, per lattice and
+storage, on ragged grids, and the collision with and without a body force on
+the same grid (the runs without one leave the source's zero terms out)."""
+import numpy as np
+import pytest
+
+import workloads as W
+from oracle import lbm as olbm
+from oracle.lattice import get as get_lattice
+from tests.parity import gpu_to_oracle_order, oracle_from_workload, rel_err
+
+pytestmark = pytest.mark.gpu
+
+SHAPES = [(19, (9, 11, 33)), (19, (8, 10, 130)), (9, (1, 13, 67))]
+# relative size of one rounding of a stored deviation (FP64 runs are held to
+# the oracle at 1e-14 in test_gpu_lbm.py)
+UNIT = {"fp32": 2.0 ** -24, "fp16dev": 2.0 ** -11, "bf16dev": 2.0 ** -8}
+
+
+def _ctx(ibl, q, shape, prec, force=(0.0, 0.0, 0.0)):
+    grid = W.grid(shape[2], shape[1], shape[0], [W.PERIODIC] * 6, body_force=force, precision=prec)
+    return ibl.from_workload({"lattice": q, "tau": 0.7, "grid": grid, "bodies": []}, init=False)
+
+
+@pytest.mark.parametrize("q,shape", SHAPES)
+@pytest.mark.parametrize("prec", list(UNIT))
+@pytest.mark.parametrize("given", ["rest", "u", "rho_u"])
+def test_init_and_readout(ibl, q, shape, prec, given):
+    lat = get_lattice(q)
+    rng = np.random.default_rng(3)
+    u = np.zeros((lat.d,) + shape) if given == "rest" else rng.uniform(-0.05, 0.05, size=(lat.d,) + shape)
+    rho = 1 + 0.02 * rng.uniform(-1, 1, size=shape) if given == "rho_u" else np.ones(shape)
+    ctx = _ctx(ibl, q, shape, prec)
+    ctx.ibl_init_fluid(rho if given == "rho_u" else None, None if given == "rest" else u)
+    perm = gpu_to_oracle_order(ibl, q)
+    f = ctx.ibl_get_populations()[perm]
+    want = olbm.equilibrium(lat, rho, u)
+    dev = np.abs(want - lat.w[:, None, None, None])
+    # each deviation is rounded to the storage once (FP16 through FP32, below
+    # 2^-24 / 2^8 in steps)
+    bound = 1.01 * UNIT[prec] * dev + (2.0 ** -32 if prec == "fp16dev" else 0.0) + 4e-17
+    assert (np.abs(f - want) <= bound).all()
+    # read-out against the stored populations themselves
+    got_rho, got_u = ctx.ibl_get_field(ibl.IBL_FIELD_RHO), ctx.ibl_get_field(ibl.IBL_FIELD_U)
+    r, m = olbm.density(f), olbm.momentum(lat, f)
+    assert np.abs(got_rho - r).max() < 1e-14
+    assert np.abs(got_u - m / r).max() < 1e-14
+    mass = ctx.ibl_mass()
+    assert abs(mass - r.sum()) < 1e-13 * r.sum()
+    assert mass == ctx.ibl_mass_noalloc(1024)
+
+
+def test_readout_of_infinite_populations(ibl):
+    q, shape = 19, (8, 8, 8)
+    lat = get_lattice(q)
+    f = np.tile(lat.w[:, None, None, None], (1,) + shape)
+    f[0, 3, 4, 5] = np.inf
+    ctx = _ctx(ibl, q, shape, "fp32")
+    ctx.ibl_set_populations(f)
+    rho = ctx.ibl_get_field(ibl.IBL_FIELD_RHO)
+    assert np.isposinf(rho[3, 4, 5]) and np.isfinite(np.delete(rho.ravel(), (3 * 8 + 4) * 8 + 5)).all()
+    assert np.isposinf(ctx.ibl_mass())
+
+
+@pytest.mark.parametrize("prec", ["fp64", "fp32", "fp16dev"])
+@pytest.mark.parametrize("force", [(0.0, 0.0, 0.0), (0.0, 1e-5, 0.0)])
+def test_collision_with_and_without_force(ibl, prec, force):
+    q, shape = 19, (9, 10, 34)
+    grid = W.grid(shape[2], shape[1], shape[0], [W.PERIODIC] * 6, body_force=force, precision=prec)
+    cfg = {"lattice": q, "tau": 0.7, "grid": grid, "bodies": []}
+    rng = np.random.default_rng(8)
+    u = rng.uniform(-0.03, 0.03, size=(3,) + shape)
+    ctx, sim = ibl.from_workload(cfg, init=False), oracle_from_workload(cfg)
+    ctx.ibl_init_fluid(None, u)
+    sim.init_fluid(u=u)
+    ctx.ibl_step(5)
+    sim.step(5)
+    # five steps: the storage's rounding of deviations up to 0.03, a few times per step
+    tol = {"fp64": 1e-13, "fp32": 5e-6, "fp16dev": 2e-2}[prec]
+    assert rel_err(ctx.ibl_get_field(ibl.IBL_FIELD_U), sim.fields()[1]) < tol
