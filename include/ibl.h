@@ -303,7 +303,10 @@ ibl_status ibl_solver_blocks(ibl_ctx* ctx, int32_t blocks);
  *           factors' inverses and one Schur block over the mesh's bounding
  *           rectangle (n_k^2 + n_k n_i^2 + n_c^2 numbers; 3D only);
  *   kind -1 (default): kind 1 when every body qualifies and the largest has
- *           at least 4096 markers, else kind 0.
+ *           at least 4096 markers, else kind 0; up to 640 markers in all the
+ *           solve with kind 0 then runs on one thread-block cluster, whose
+ *           size follows from the marker count (ibl_solver_blocks has no
+ *           effect on it).
  * A change of kind takes effect at the next step and restarts the solver's
  * warm start.  IBL_EINVAL at the next step if kind 1 is asked for bodies
  * that do not qualify.
@@ -320,18 +323,20 @@ ibl_status ibl_solver_preconditioner(ibl_ctx* ctx, int32_t kind, int32_t residen
  * runs, and the band tiles collide after the spreading; 2 = serial split:
  * after the IB chain, the cells outside the band collide in a kernel without
  * the band lookup on every SM, then the band tiles; -1 (default) = split on
- * grids of at least 2^20 cells with at most 8192 markers, else 0.  All give
+ * grids of at least 2^18 cells with at most 8192 markers, else 0.  All give
  * bitwise the same populations and forces (every cell runs the same
  * arithmetic). */
 ibl_status ibl_set_overlap(ibl_ctx* ctx, int32_t mode);
 
 /* Launch shape of the one-kernel collide (the kernel of steps without the
  * split, see ibl_set_overlap): thread blocks of bx x by threads, bx in
- * {32, 64, 128, 256}, bx * by <= 256 (default 64 x 2).  With 16-bit storage
+ * {32, 64, 128, 256}, bx * by <= 256 (until it is called: 64 x 2, or 32 x 4 where
+ * rows fit it better, or 32 x 1 on grids of few cells).  With 16-bit storage
  * and nx even, each thread takes the two x-adjacent cells (x, x + 1), whose
  * collisions run as packed FP32 pairs: pairs = 3 (default) walks 8 z-planes
  * per thread, the next plane's loads in flight while the current one
- * collides; pairs = 1 one plane per thread; pairs = 2 blocks of 64 x 4
+ * collides (until it is called, grids that leave too few threads take one plane
+ * per thread); pairs = 1 one plane per thread; pairs = 2 blocks of 64 x 4
  * threads walk 16 z-planes of 128 x 4 cells, the next plane's source rows
  * arriving in shared memory by bulk asynchronous copies (D3Q19 with nx a
  * multiple of 8; otherwise as 1); pairs = 0 one cell per thread.  Every

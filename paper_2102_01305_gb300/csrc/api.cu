@@ -371,7 +371,7 @@ ibl_status ibl_step(ibl_ctx* c, int64_t n) {
   const bool with_ib = c->m_total > 0;
   // split step: the cells outside the IB band collide on a second stream
   // while the IB chain runs; the band tiles collide after the spreading
-  const bool split = with_ib && (c->overlap == 1 || (c->overlap < 0 && c->N >= (1LL << 20) &&
+  const bool split = with_ib && (c->overlap == 1 || (c->overlap < 0 && c->N >= SPLIT_MIN_CELLS &&
                                                      c->m_total <= SPLIT_MAX_MARKERS));
   // serial split (on request): the IB chain on every SM, then the cells
   // outside the band (the persistent kernel without the band lookup, every
@@ -487,6 +487,7 @@ ibl_status ibl_set_collide_shape(ibl_ctx* c, int32_t bx, int32_t by, int32_t pai
   if (!c) return IBL_EINVAL;
   if (!(bx == 32 || bx == 64 || bx == 128 || bx == 256) || by < 1 || bx * by > 256 || pairs < 0 || pairs > 3)
     return fail(c, IBL_EINVAL, "collide shape: bx in {32, 64, 128, 256}, by >= 1, bx * by <= 256, pairs 0 .. 3");
+  c->collide_auto = false;
   c->collide_bx = bx;
   c->collide_by = by;
   c->collide_pairs = pairs;

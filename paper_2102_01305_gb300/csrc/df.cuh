@@ -137,13 +137,27 @@ __device__ __forceinline__ void acc_fma_ff(dfacc& a, float x, float y) {
 __device__ __forceinline__ df acc_value(dfacc a) { return fast_two_sum(a.s, a.c); }
 
 // Butterfly sum over groups of `width` lanes in a fixed order (every lane of
-// a group ends with the same total).
+// a group ends with the same total).  The trees are loops: unrolled, their
+// 24 instructions a level dominated the code of the latency-bound solve
+// kernels, which run every instruction once an iteration and wait for its
+// fetch.  Sums of several values share a loop, so that their chains overlap.
+__device__ __forceinline__ df df_shfl_xor(df v, int o) {
+  return df_make(__shfl_xor_sync(0xffffffffu, v.hi, o), __shfl_xor_sync(0xffffffffu, v.lo, o));
+}
 __device__ __forceinline__ df df_warp_sum(df v, int width = 32) {
-  for (int o = width >> 1; o > 0; o >>= 1) {
-    const df w = df_make(__shfl_xor_sync(0xffffffffu, v.hi, o), __shfl_xor_sync(0xffffffffu, v.lo, o));
-    v = df_add(v, w);
-  }
+#pragma unroll 1
+  for (int o = width >> 1; o > 0; o >>= 1) v = df_add(v, df_shfl_xor(v, o));
   return v;
 }
+template <int N>
+__device__ __forceinline__ void df_warp_sums(df (&v)[N], int width = 32) {
+#pragma unroll 1
+  for (int o = width >> 1; o > 0; o >>= 1) {
+#pragma unroll
+    for (int c = 0; c < N; ++c) v[c] = df_add(v[c], df_shfl_xor(v[c], o));
+  }
+}
+// a / b as one shared function (for the same reason).
+static __device__ __noinline__ df df_div_call(df a, df b) { return df_div(a, b); }
 
 }  // namespace ibl

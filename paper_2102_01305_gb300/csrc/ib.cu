@@ -39,6 +39,11 @@ namespace ibl {
 constexpr int MAX_BODIES = 16;
 constexpr int GJ_NB = 64;          // Gauss-Jordan pivot block
 constexpr int PCG_MAX_ITERS = 200;
+// Marker sets whose kinematics and band run on one cluster (at 3152 markers 34 us
+// between events a step, 41 as separate kernels), and those whose solve does (an iteration takes 3.9 us at 68 markers, 7.6 at 520 and 18 at 1140,
+// where G and M no longer fit the shared memory; k_pcg 12.4, 13.2 and 13.7).
+constexpr int FRONT_MARKERS = 4096;
+constexpr int CLUSTER_MARKERS = 640;
 // relative preconditioned residual (the spread field's A-norm error) per
 // storage precision, under the field error the storage itself accumulates:
 // FP32 runs sit at field errors of ~2e-6 against the FP64 reference after
@@ -83,22 +88,31 @@ __device__ __forceinline__ int wrap(int v, int n) {
   return v;
 }
 
-// One thread per (marker, axis): the axis's position, wall velocity, stencil
-// base and weights (the rotation is recomputed by each of the three threads,
-// which is cheaper than serialising the three stencils on one thread).
-__global__ void k_kinematics(BodyTable bt, int m_total, const int* __restrict__ body_of,
-                             const double* __restrict__ X0, const double* __restrict__ Xp,
-                             const double* __restrict__ Up, double* __restrict__ X,
-                             double* __restrict__ U, int* __restrict__ base,
-                             df* __restrict__ wts, double t, Geo geo, int* status) {
-  const int gid = blockIdx.x * blockDim.x + threadIdx.x;
-  const int l = gid / 3, a = gid - 3 * (gid / 3);
-  if (l >= m_total) return;
-  const BodyDev& B = bt.b[body_of[l]];
-  double x, u;
+// Position, wall velocity, stencil bases and weights of marker l.  FP64
+// instructions (1.7 a clock and SM) bound it, so the rotation is formed once for
+// the three axes, the stencil base comes from integer arithmetic, and the
+// weights of runs that store 32 or 16 bits from double-float arithmetic
+// (axis_stencil).
+struct MotionArgs {
+  const int* body_of;
+  const double* X0;
+  const double* Xp;
+  const double* Up;
+  double* X;
+  double* U;
+  int* base;
+  df* wts;
+  int* status;
+};
+template <bool EXACT64>
+__device__ __forceinline__ void move_marker(const BodyTable& bt, int l, const MotionArgs& M, const Geo& geo) {
+  const BodyDev& B = bt.b[M.body_of[l]];
+  double x[3], u[3];
   if (B.prescribed) {
-    x = Xp[3 * l + a];
-    u = Up[3 * l + a];
+    for (int a = 0; a < 3; ++a) {
+      x[a] = M.Xp[3 * l + a];
+      u[a] = M.Up[3 * l + a];
+    }
   } else {
     // per-body motion state of this step (formed on the host): A, A', alpha', cos, sin, e_s
     const double* st = B.st;
@@ -106,40 +120,45 @@ __global__ void k_kinematics(BodyTable bt, int m_total, const int* __restrict__ 
     const double es[3] = {st[5], st[6], 0.0};
     const double* e = B.axis;
     double d[3];
-    for (int k = 0; k < 3; ++k) d[k] = X0[3 * l + k] - B.hinge[k];
+    for (int k = 0; k < 3; ++k) d[k] = M.X0[3 * l + k] - B.hinge[k];
     // Rodrigues: r = d cos + (e x d) sin + e (e.d)(1 - cos)
     const double ed = e[0] * d[0] + e[1] * d[1] + e[2] * d[2];
     const double exd[3] = {e[1] * d[2] - e[2] * d[1], e[2] * d[0] - e[0] * d[2],
                            e[0] * d[1] - e[1] * d[0]};
     double r[3];
     for (int k = 0; k < 3; ++k) r[k] = d[k] * c + exd[k] * s + e[k] * ed * (1.0 - c);
-    const int a1 = a == 2 ? 0 : a + 1, a2 = a == 0 ? 2 : a - 1;
-    const double exr = e[a1] * r[a2] - e[a2] * r[a1];
-    x = B.origin[a] + B.hinge[a] + r[a] + A * es[a];
-    u = Ad * es[a] + ald * exr;
+    const double exr[3] = {e[1] * r[2] - e[2] * r[1], e[2] * r[0] - e[0] * r[2], e[0] * r[1] - e[1] * r[0]};
+    for (int a = 0; a < 3; ++a) {
+      x[a] = B.origin[a] + B.hinge[a] + r[a] + A * es[a];
+      u[a] = Ad * es[a] + ald * exr[a];
+    }
   }
-  if (a >= geo.D) {
-    X[3 * l + a] = 0.0;
-    U[3 * l + a] = 0.0;
-    base[3 * l + a] = 0;
-    wts[12 * l + 4 * a + 0] = df_make(1.f, 0.f);
-    wts[12 * l + 4 * a + 1] = df_make(0.f, 0.f);
-    wts[12 * l + 4 * a + 2] = df_make(0.f, 0.f);
-    wts[12 * l + 4 * a + 3] = df_make(0.f, 0.f);
-    return;
+  bool ok = true;
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    const bool in = a < geo.D;
+    df w[4] = {df_make(1.f, 0.f), df_make(0.f, 0.f), df_make(0.f, 0.f), df_make(0.f, 0.f)};
+    int b0 = 0;
+    if (in) ok = axis_stencil<EXACT64>(x[a], geo.n[a], geo.per[a] != 0, b0, w) && ok;
+    M.X[3 * l + a] = in ? x[a] : 0.0;
+    M.U[3 * l + a] = in ? u[a] : 0.0;
+    M.base[3 * l + a] = b0;
+    for (int k = 0; k < 4; ++k) M.wts[12 * l + 4 * a + k] = w[k];
   }
-  X[3 * l + a] = x;
-  U[3 * l + a] = u;
-  int b0;
-  double w[4];
-  if (!stencil_axis(x, geo.n[a], geo.per[a] != 0, b0, w)) atomicOr(status, ST_OVERFLOW);
-  for (int k = 0; k < 4; ++k) wts[12 * l + 4 * a + k] = df_from_double(w[k]);
-  base[3 * l + a] = b0;
+  if (!ok) atomicOr(M.status, ST_OVERFLOW);
+}
+
+template <bool EXACT64>
+__global__ void k_kinematics(BodyTable bt, int m_total, MotionArgs M, Geo geo) {
+  const int l = blockIdx.x * blockDim.x + threadIdx.x;
+  if (l < m_total) move_marker<EXACT64>(bt, l, M, geo);
 }
 
 // ------------------------------------------------------------------ band tiles
+// log2 of a tile's extent on axis a (16 x 4 x 4 cells in 3D, 16 x 16 in 2D)
+__device__ __forceinline__ int tile_log2(int D, int a) { return a == 0 || D == 2 ? 4 : 2; }
 __device__ __forceinline__ int tile_of(const Geo& g, int nx, int ny, int nz) {
-  return ((nz / g.tg.tz) * g.tg.nty + (ny / g.tg.ty)) * g.tg.ntx + (nx / g.tg.tx);
+  return ((nz >> (g.D == 3 ? 2 : 0)) * g.tg.nty + (ny >> tile_log2(g.D, 1))) * g.tg.ntx + (nx >> 4);
 }
 
 // Tiles touched by marker l's stencil (at most 2 per axis); returns the count.
@@ -147,11 +166,10 @@ __device__ int touched_tiles(const Geo& g, const int* b, int out[8]) {
   int tl[3][2], cnt[3];
   for (int a = 0; a < 3; ++a) {
     if (a >= g.D) { tl[a][0] = 0; cnt[a] = 1; continue; }
-    const int ext = a == 0 ? g.tg.tx : (a == 1 ? g.tg.ty : g.tg.tz);
     cnt[a] = 0;
     for (int k = 0; k < 4; ++k) {
       const int node = g.per[a] ? wrap(b[a] + k, g.n[a]) : b[a] + k;
-      const int t = node / ext;
+      const int t = node >> tile_log2(g.D, a);
       bool seen = false;
       for (int j = 0; j < cnt[a]; ++j) seen |= (tl[a][j] == t);
       if (!seen && cnt[a] < 2) tl[a][cnt[a]++] = t;
@@ -221,6 +239,70 @@ __global__ void k_append_markers(int m_total, const int* __restrict__ base, Geo 
   else atomicOr(status, ST_OVERFLOW);
 }
 
+// The same for marker sets up to FRONT_MARKERS in one kernel on one cluster:
+// kinematics, the last band's tiles back to -1, the tiles of this step's band,
+// and, only when the assembly will read them, the tiles' marker lists.  As five
+// kernels and three fills of a few microseconds each, they took 33 us (37) of a
+// step at 63 (520) markers between events, 17 (16) now.  counts[cur]
+// is this step's slot count (zero on entry), counts[1 - cur] the last one's.
+struct FrontArgs {
+  int m, cap, cur, use_tiles;
+  int* tile_slot;
+  int* slot_tile;
+  int* counts;
+  int* tile_mcount;
+  int* tile_markers;
+  int* mixed;                 // [0] this step, [1] always: the assembly searches the tiles' lists
+  double* rowsum_max;         // per body, cleared
+};
+template <bool EXACT64>
+__global__ void __launch_bounds__(512, 1) k_ib_front(BodyTable bt, MotionArgs M, Geo g, FrontArgs F) {
+  cg::cluster_group cl = cg::this_cluster();
+  const int gtid = blockIdx.x * blockDim.x + threadIdx.x, nth = gridDim.x * blockDim.x;
+  const int old = min(F.counts[1 - F.cur], F.cap);
+  for (int s = gtid; s < old; s += nth) F.tile_slot[F.slot_tile[s]] = -1;
+  if (gtid < MAX_BODIES) F.rowsum_max[gtid] = 0.0;
+  if (gtid == 0) *F.mixed = F.use_tiles;
+  // markers dealt to the blocks in turn, so that every SM's FP64 units work
+  for (int l = threadIdx.x * gridDim.x + blockIdx.x; l < F.m; l += nth) move_marker<EXACT64>(bt, l, M, g);
+  cl.sync();
+  // a tile's first marker claims it (-2 - body) and takes a slot
+  for (int e = gtid; e < 8 * F.m; e += nth) {
+    const int l = e >> 3, i = e & 7;
+    int t[8];
+    if (i >= touched_tiles(g, M.base + 3 * l, t)) continue;
+    const int mine = -2 - M.body_of[l];
+    const int prev = atomicCAS(&F.tile_slot[t[i]], -1, mine);
+    if (prev == -1) {
+      const int s = atomicAdd(&F.counts[F.cur], 1);
+      if (s < F.cap) {
+        F.slot_tile[s] = t[i];
+        F.tile_mcount[s] = 0;
+      } else {
+        atomicOr(M.status, ST_OVERFLOW);   // the tile keeps no slot
+      }
+    } else if (prev != mine) {
+      *F.mixed = 1;   // two bodies' stencils share a tile
+    }
+  }
+  cl.sync();
+  const int cnt = min(__ldcg(&F.counts[F.cur]), F.cap);
+  for (int s = gtid; s < cnt; s += nth) F.tile_slot[__ldcg(&F.slot_tile[s])] = s;
+  if (gtid == 0) F.counts[1 - F.cur] = 0;
+  if (!__ldcg(F.mixed) && !__ldcg(F.mixed + 1)) return;
+  cl.sync();
+  for (int e = gtid; e < 8 * F.m; e += nth) {
+    const int l = e >> 3, i = e & 7;
+    int t[8];
+    if (i >= touched_tiles(g, M.base + 3 * l, t)) continue;
+    const int s = __ldcg(&F.tile_slot[t[i]]);
+    if (s < 0) continue;
+    const int pos = atomicAdd(&F.tile_mcount[s], 1);
+    if (pos < TILE_MARKER_CAP) F.tile_markers[s * TILE_MARKER_CAP + pos] = l;
+    else atomicOr(M.status, ST_OVERFLOW);
+  }
+}
+
 // rho_l and u*_l (Eq. 17) gathered straight from the populations of each
 // stencil node (the same pull, face rules and moment arithmetic as the
 // collision), FP64 accumulation; B = U_B - u*_l (Eq. 19).  One warp per
@@ -248,15 +330,16 @@ __device__ __forceinline__ void interpolate_body(int vblock, int m_total, const 
       if (g.per[a]) node[a] = wrap(node[a], g.n[a]);
     df wt = df_mul(w[i], w[4 + j]);
     if (g.D == 3) wt = df_mul(wt, w[8 + q]);
-    const long long cell = ((long long)node[2] * p.ny + node[1]) * p.nx + node[0];
     R drho, u[3];
-    node_moments<Q, T, PULL>(src, node[0], node[1], node[2], cell, p, drho, u);
+    node_moments_fast<Q, T, PULL>(src, node[0], node[1], node[2], p, drho, u);
     acc_fma(acc[0], wt, df_from_float(1.f));
     acc_fma(acc[0], wt, to_df(drho));
     for (int c = 0; c < 3; ++c) acc_fma(acc[1 + c], wt, to_df(u[c]));
   }
   df v[4];
-  for (int c = 0; c < 4; ++c) v[c] = df_warp_sum(acc_value(acc[c]));
+#pragma unroll
+  for (int c = 0; c < 4; ++c) v[c] = acc_value(acc[c]);
+  df_warp_sums(v);
   if (lane == 0) {
     rho_l[l] = df_to_double(v[0]);
     for (int a = 0; a < 3; ++a) B[3 * l + a] = (a < g.D) ? U[3 * l + a] - df_to_double(v[1 + a]) : 0.0;
@@ -578,23 +661,23 @@ __device__ __forceinline__ void trace_mark(const PcgArgs& A, int slot) {
 // Fixed-order block sum of three doubles per warp (lane 0 holds them); the
 // totals are returned to every thread.
 __device__ void block_total3(double v[3], double* sh) {
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, warps = blockDim.x >> 5;
   __syncthreads();
   if (lane == 0)
     for (int c = 0; c < 3; ++c) sh[3 * wid + c] = v[c];
   __syncthreads();
   if (threadIdx.x < 32) {
     for (int c = 0; c < 3; ++c) {
-      double t = threadIdx.x < PCG_WARPS ? sh[3 * threadIdx.x + c] : 0.0;
+      double t = threadIdx.x < warps ? sh[3 * threadIdx.x + c] : 0.0;
       for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
       v[c] = t;
     }
   }
   __syncthreads();
   if (threadIdx.x == 0)
-    for (int c = 0; c < 3; ++c) sh[3 * PCG_WARPS + c] = v[c];
+    for (int c = 0; c < 3; ++c) sh[3 * warps + c] = v[c];
   __syncthreads();
-  for (int c = 0; c < 3; ++c) v[c] = sh[3 * PCG_WARPS + c];
+  for (int c = 0; c < 3; ++c) v[c] = sh[3 * warps + c];
 }
 
 // Fixed-order block sum of one double per warp (lane 0 holds it); the total
@@ -662,26 +745,25 @@ __device__ void block_partial3(df v, df* sh, df* out) {
 
 // Grid total of one double-float partial (slot `slot` of every block), for
 // one warp: each lane issues all of its loads at once (one memory round
-// trip), adds its blocks in a fixed pairwise tree, then a butterfly; every
-// lane ends with the total.
+// trip), adds its blocks in order, then a butterfly; every lane ends with the
+// total.
 __device__ __forceinline__ df grid_total_df(const df* red, int slot) {
   constexpr int U = MAX_PCG_BLOCKS / 32;
-  const int lane = threadIdx.x & 31;
+  const int lane = threadIdx.x & 31, n = ((int)gridDim.x + 31) >> 5;
   float2 v[U];
 #pragma unroll
   for (int u = 0; u < U; ++u) {
     const int b = lane + 32 * u;
     v[u] = b < (int)gridDim.x ? __ldcg(reinterpret_cast<const float2*>(red + b * 8 + slot)) : make_float2(0.f, 0.f);
   }
-  // pairwise tree over the lane's blocks (depth log2 U instead of U)
-  df t[U];
+  // the lane's own blocks in order, then a butterfly
+  df t = df_make(v[0].x, v[0].y);
 #pragma unroll
-  for (int u = 0; u < U; ++u) t[u] = df_make(v[u].x, v[u].y);
-#pragma unroll
-  for (int w = U / 2; w >= 1; w >>= 1)
-#pragma unroll
-    for (int u = 0; u < w; ++u) t[u] = df_add(t[u], t[u + w]);
-  return df_warp_sum(t[0]);
+  for (int u = 1; u < U; ++u) {
+    if (u >= n) break;
+    t = df_add(t, df_make(v[u].x, v[u].y));
+  }
+  return df_warp_sum(t);
 }
 
 // Row stride of a body's dense preconditioner: padded to 4 floats so rows
@@ -824,6 +906,7 @@ __device__ __forceinline__ void precond_pair(const PcgArgs& A, int p, const floa
     b0 = fmaf(m1.z, x1.z, b0); b1 = fmaf(m1.z, x1.w, b1); b2 = fmaf(m1.z, x2.x, b2);
     b0 = fmaf(m1.w, x2.y, b0); b1 = fmaf(m1.w, x2.z, b1); b2 = fmaf(m1.w, x2.w, b2);
   }
+#pragma unroll 1
   for (int off = 16; off > 0; off >>= 1) {
     a0 += __shfl_xor_sync(0xffffffffu, a0, off);
     a1 += __shfl_xor_sync(0xffffffffu, a1, off);
@@ -860,6 +943,7 @@ constexpr size_t PCG_SMEM_MAX = 224 * 1024;
 // [ck0, ck1).  Ag points at the tile's first A row; Bg at B's row 0 (its
 // columns are absolute).  Inputs are staged in shared memory before any
 // output is written, so out may alias A or B within the tile.
+template <int NT>   // threads of the block
 __device__ __noinline__ void tile_gemm(float* out, int ldo, const float* Ag, int lda, const float* Bg, int ldb, int i0,
                           int j0, int nr, int nc, int K, float alpha, bool acc, int sk0, int sk1, int ck0,
                           int ck1, float* sm) {
@@ -871,11 +955,11 @@ __device__ __noinline__ void tile_gemm(float* out, int ldo, const float* Ag, int
   // except at ragged edges, where the group falls back to masked scalar
   // loads); lda, ldb and the tile origins are multiples of 4 floats, so full
   // groups are 16-byte aligned.
-  for (int u0 = 0; u0 < 2048 / PCG_THREADS; u0 += 2) {
+  for (int u0 = 0; u0 < 2048 / NT; u0 += 2) {
     float4 av[2], bv[2];
 #pragma unroll
     for (int u = 0; u < 2; ++u) {
-      const int f = threadIdx.x + (u0 + u) * PCG_THREADS;
+      const int f = threadIdx.x + (u0 + u) * NT;
       const int r = f >> 4, q4 = (f & 15) << 2;
       if (r < nr && q4 + 3 < K) {
         av[u] = __ldcg(reinterpret_cast<const float4*>(Ag + (long long)r * lda + q4));
@@ -895,7 +979,7 @@ __device__ __noinline__ void tile_gemm(float* out, int ldo, const float* Ag, int
     }
 #pragma unroll
     for (int u = 0; u < 2; ++u) {
-      const int f = threadIdx.x + (u0 + u) * PCG_THREADS;
+      const int f = threadIdx.x + (u0 + u) * NT;
       const int r = f >> 4, q4 = (f & 15) << 2;
       As[(q4 + 0) * GS + r] = av[u].x;
       As[(q4 + 1) * GS + r] = av[u].y;
@@ -906,9 +990,9 @@ __device__ __noinline__ void tile_gemm(float* out, int ldo, const float* Ag, int
     }
   }
   __syncthreads();
-  // 32 x 32 groups of 4 x 4 outputs, PCG_THREADS / 32 row groups at a time
+  // 32 x 32 groups of 4 x 4 outputs, NT / 32 row groups at a time
   const int tx = threadIdx.x & 31;
-  for (int ty = threadIdx.x >> 5; ty < 32; ty += PCG_THREADS / 32) {
+  for (int ty = threadIdx.x >> 5; ty < 32; ty += NT / 32) {
     float a4[4][4];
     for (int u = 0; u < 4; ++u)
       for (int v = 0; v < 4; ++v) a4[u][v] = 0.f;
@@ -1006,7 +1090,8 @@ __device__ __forceinline__ int first_tile(int done) {
   return t < 0 ? t + (int)gridDim.x : t;
 }
 
-__device__ __noinline__ void gj_invert(const PcgArgs& A, cg::grid_group& grid, float* sm) {
+template <int NT, class Group>   // Group: the blocks that share the work, a grid or a cluster
+__device__ __noinline__ void gj_invert(const PcgArgs& A, Group& grid, float* sm) {
   int maxnb = 0;
   for (int b = 0; b < A.nbodies; ++b) {
     const int mb = A.boff[b + 1] - A.boff[b];
@@ -1043,7 +1128,7 @@ __device__ __noinline__ void gj_invert(const PcgArgs& A, cg::grid_group& grid, f
         const int nt = (mb + GT - 1) / GT;
         for (int t = first_tile(done); t < nt; t += gridDim.x) {
           const int j0 = t * GT;
-          tile_gemm(Mb, ld, Mb + (long long)k0 * ld + k0, ld, Mb + (long long)k0 * ld, ld, k0, j0, kn,
+          tile_gemm<NT>(Mb, ld, Mb + (long long)k0 * ld + k0, ld, Mb + (long long)k0 * ld, ld, k0, j0, kn,
                     min(GT, mb - j0), kn, 1.0f, false, -1, -1, k0, k0 + kn, sm);
         }
         done += nt;
@@ -1062,7 +1147,7 @@ __device__ __noinline__ void gj_invert(const PcgArgs& A, cg::grid_group& grid, f
         const int nt = (mb + GT - 1) / GT;
         for (int t = first_tile(done); t < nt * nt; t += gridDim.x) {
           const int i0 = (t / nt) * GT, j0 = (t % nt) * GT;
-          tile_gemm(Mb, ld, Mb + (long long)i0 * ld + k0, ld, Mb + (long long)k0 * ld, ld, i0, j0,
+          tile_gemm<NT>(Mb, ld, Mb + (long long)i0 * ld + k0, ld, Mb + (long long)k0 * ld, ld, i0, j0,
                     min(GT, mb - i0), min(GT, mb - j0), kn, -1.0f, true, k0, k0 + kn, k0, k0 + kn, sm);
         }
         done += nt * nt;
@@ -1081,7 +1166,7 @@ __device__ __noinline__ void gj_invert(const PcgArgs& A, cg::grid_group& grid, f
         const int nt = (mb + GT - 1) / GT;
         for (int t = first_tile(done); t < nt; t += gridDim.x) {
           const int i0 = t * GT;
-          tile_gemm(Mb, ld, Mb + (long long)i0 * ld + k0, ld, Mb + (long long)k0 * ld, ld, i0, k0,
+          tile_gemm<NT>(Mb, ld, Mb + (long long)i0 * ld + k0, ld, Mb + (long long)k0 * ld, ld, i0, k0,
                     min(GT, mb - i0), kn, kn, -1.0f, false, k0, k0 + kn, -1, -1, sm);
         }
         done += nt;
@@ -1090,6 +1175,34 @@ __device__ __noinline__ void gj_invert(const PcgArgs& A, cg::grid_group& grid, f
     grid.sync();
     if (kb == 0) trace_mark(A, 7);
   }
+}
+
+// Dense rebuild: M_b <- (G_b + sigma_b I)^-1 in FP32 for every body.
+template <int NT, class Group>
+__device__ void rebuild_dense(const PcgArgs& A, Group& grid, float* sm) {
+  const int gtid = blockIdx.x * blockDim.x + threadIdx.x, nthreads = gridDim.x * blockDim.x;
+  if (gtid == 0 && !A.refresh) A.info[3] += 1;   // early rebuilds (a slow previous solve)
+  for (int b = 0; b < A.nbodies; ++b) {
+    const int mb = A.boff[b + 1] - A.boff[b];
+    const long long tot = (long long)mb * precond_ld(mb);
+    for (long long e = gtid; e < tot; e += nthreads) A.M[A.poff[b] + e] = 0.f;
+  }
+  grid.sync();
+  for (int l = gtid; l < A.m_total; l += nthreads) {
+    const int b = A.body_of[l];
+    const int o = A.boff[b], mb = A.boff[b + 1] - o, ld = precond_ld(mb);
+    const double sigma = 1e-6 * __longlong_as_double((long long)A.rowsum_max[b]);
+    float* Mb = A.M + A.poff[b];
+    for (int j = 0; j < A.Gnnz[l]; ++j) {
+      const int k = A.Gcol[(long long)l * G_MAXNNZ + j];
+      if (A.body_of[k] != b) continue;   // block-Jacobi over bodies
+      double v = df_to_double(A.Gv[(long long)l * G_MAXNNZ + j]);
+      if (k == l) v += sigma;
+      Mb[(long long)(l - o) * ld + (k - o)] = (float)v;
+    }
+  }
+  grid.sync();
+  gj_invert<NT>(A, grid, sm);
 }
 
 // Stages A-G of the separable preconditioner (sep.cuh) for all bodies and
@@ -1112,6 +1225,46 @@ __device__ void sep_apply(const PcgArgs& A, cg::grid_group& grid, const SepIn& i
     }
     grid.sync();
     if (trace) trace_mark(A, marks[st]);
+  }
+}
+
+// The end of a solve, after the whole solution is in A.wd and visible to every
+// block: F_w = -sum_l 2 rho_l w_l per body (Eq. 26 x ds, Sec. 3.7), block b mod
+// gridDim reducing body b in a fixed order (lane-strided FP64 sums, fixed
+// shuffle tree, warp order), and the solver's bookkeeping.
+__device__ void finish_solve(const PcgArgs& A, int it, bool done, bool rebuild, const df* s_scale, const df* s_rz,
+                             double* shd) {
+  for (int b = blockIdx.x; b < A.nbodies; b += gridDim.x) {
+    double v[3] = {0, 0, 0};
+    for (int l = A.boff[b] + threadIdx.x; l < A.boff[b + 1]; l += blockDim.x)
+      for (int c = 0; c < 3; ++c) {
+        const double f = 2.0 * A.rho_l[l] * df_to_double(A.wd[3 * l + c]);   // force on the fluid
+        A.mforce[3 * l + c] = f;
+        v[c] += f;
+      }
+    for (int o = 16; o > 0; o >>= 1)
+      for (int c = 0; c < 3; ++c) v[c] += __shfl_xor_sync(0xffffffffu, v[c], o);
+    block_total3(v, shd);
+    if (threadIdx.x == 0) {
+      double* h = A.hist + ((long long)b * HIST_LEN + (A.step % HIST_LEN)) * 3;
+      for (int c = 0; c < 3; ++c) h[c] = -v[c];   // force on the body
+    }
+  }
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    double rel = 0.0;
+    for (int c = 0; c < A.D; ++c)
+      if (s_scale[c].hi > 0.f) rel = fmax(rel, sqrt(fmax(df_to_double(s_rz[c]), 0.0) / df_to_double(s_scale[c])));
+    A.info[0] = it;
+    if (rebuild) {
+      A.info[4] = it;
+      A.info[5] = 0;
+    } else {
+      A.info[5] = min(A.info[5] + max(it - max(A.info[4], REBUILD_ITERS_OK), 0), 1 << 30);
+    }
+    A.info[1] = (A.info[5] > A.rebuild_excess || !done) ? 1 : 0;
+    A.info[2] = done ? 1 : 0;
+    *A.res = rel;
+    if (!done) atomicOr(A.status, ST_NOTCONV);
   }
 }
 
@@ -1140,30 +1293,7 @@ __global__ void __launch_bounds__(PCG_THREADS, 1) k_pcg(PcgArgs A) {
   // the separable factors are rebuilt by their own kernel on the host's
   // schedule only (sep_launch), so early requests apply to the dense path
   const bool rebuild = A.refresh || (!A.sep_on && A.info[1]);
-  if (rebuild && !A.sep_on) {
-    if (gtid == 0 && !A.refresh) A.info[3] += 1;   // early rebuilds (a slow previous solve)
-    for (int b = 0; b < A.nbodies; ++b) {
-      const int mb = A.boff[b + 1] - A.boff[b];
-      const long long tot = (long long)mb * precond_ld(mb);
-      for (long long e = gtid; e < tot; e += nthreads) A.M[A.poff[b] + e] = 0.f;
-    }
-    grid.sync();
-    for (int l = gtid; l < m; l += nthreads) {
-      const int b = A.body_of[l];
-      const int o = A.boff[b], mb = A.boff[b + 1] - o, ld = precond_ld(mb);
-      const double sigma = 1e-6 * __longlong_as_double((long long)A.rowsum_max[b]);
-      float* Mb = A.M + A.poff[b];
-      for (int j = 0; j < A.Gnnz[l]; ++j) {
-        const int k = A.Gcol[(long long)l * G_MAXNNZ + j];
-        if (A.body_of[k] != b) continue;   // block-Jacobi over bodies
-        double v = df_to_double(A.Gv[(long long)l * G_MAXNNZ + j]);
-        if (k == l) v += sigma;
-        Mb[(long long)(l - o) * ld + (k - o)] = (float)v;
-      }
-    }
-    grid.sync();
-    gj_invert(A, grid, sm);
-  }
+  if (rebuild && !A.sep_on) rebuild_dense<PCG_THREADS>(A, grid, sm);
   // the preconditioner is applied to row pairs (2p, 2p + 1), pair p owned by
   // block p mod gridDim, warp (p / gridDim) mod 32; this block's pairs
   // (jp-th: p = blockIdx.x + gridDim.x jp) stay in shared memory, rows 2jp
@@ -1223,11 +1353,12 @@ __global__ void __launch_bounds__(PCG_THREADS, 1) k_pcg(PcgArgs A) {
         acc_fma(a2, v, A.wd[3 * k + 2]);
       }
     }
-    const df g0 = df_warp_sum(acc_value(a0)), g1 = df_warp_sum(acc_value(a1)), g2 = df_warp_sum(acc_value(a2));
+    df gw[3] = {acc_value(a0), acc_value(a1), acc_value(a2)};
+    df_warp_sums(gw);
     if (lane < 3) {
       const int c = lane;
       const int vi = A.voff[A.body_of[l]] + 3 * (l - A.boff[A.body_of[l]]) + c;
-      const df gx = c == 0 ? g0 : (c == 1 ? g1 : g2);
+      const df gx = c == 0 ? gw[0] : (c == 1 ? gw[1] : gw[2]);
       const df b = df_from_double(A.B[3 * l + c]);
       const df r = df_sub(b, gx);
       A.rd[3 * l + c] = r;
@@ -1380,14 +1511,14 @@ __global__ void __launch_bounds__(PCG_THREADS, 1) k_pcg(PcgArgs A) {
             acc_fma_f(a2, v, zs[3 * k + 2]);
           }
         }
-        const df gz0 = df_warp_sum(acc_value(a0), 8), gz1 = df_warp_sum(acc_value(a1), 8);
-        const df gz2 = df_warp_sum(acc_value(a2), 8);
+        df gz3[3] = {acc_value(a0), acc_value(a1), acc_value(a2)};
+        df_warp_sums(gz3, 8);
         df contrib = dzero;
         if (l < m && sl < 3) {
           const int c = sl;
           const int bd = A.body_of[l];
           const int vi = A.voff[bd] + 3 * (l - A.boff[bd]) + c;
-          const df gz = c == 0 ? gz0 : (c == 1 ? gz1 : gz2);
+          const df gz = c == 0 ? gz3[0] : (c == 1 ? gz3[1] : gz3[2]);
           const df beta = s_beta[c];
           const df pl = df_add(df_from_float(z0), df_mul(beta, p0));
           const df ap = df_add(gz, df_mul(beta, ap0));
@@ -1398,6 +1529,7 @@ __global__ void __launch_bounds__(PCG_THREADS, 1) k_pcg(PcgArgs A) {
           contrib = df_mul(pl, ap);
         }
         // lane c < 3 gathers component c of the warp's four rows, in row order
+#pragma unroll 1
         for (int r = 0; r < 4; ++r) {
           const int src = 8 * r + (lane & 7);
           const df v = df_make(__shfl_sync(0xffffffffu, contrib.hi, src), __shfl_sync(0xffffffffu, contrib.lo, src));
@@ -1416,7 +1548,7 @@ __global__ void __launch_bounds__(PCG_THREADS, 1) k_pcg(PcgArgs A) {
       const int c = wib;
       const df pAp = grid_total_df(A.red, c);
       if (lane == 0) {
-        const df a = (pAp.hi > 0.f && s_rz[c].hi > 0.f) ? df_div(s_rz[c], pAp) : dzero;
+        const df a = (pAp.hi > 0.f && s_rz[c].hi > 0.f) ? df_div_call(s_rz[c], pAp) : dzero;
         s_alpha[c] = a;
         s_alphaf[c] = a.hi;
       }
@@ -1495,7 +1627,7 @@ __global__ void __launch_bounds__(PCG_THREADS, 1) k_pcg(PcgArgs A) {
       const df rzn = grid_total_df(A.red, 3 + c);
       if (lane == 0) {
         const df prev = s_rz[c];
-        s_beta[c] = prev.hi > 0.f ? df_div(rzn, prev) : dzero;
+        s_beta[c] = prev.hi > 0.f ? df_div_call(rzn, prev) : dzero;
         s_rz[c] = rzn;
         s_conv[c] = (c >= A.D || !df_greater(rzn, s_stop[c])) ? 1 : 0;
       }
@@ -1505,9 +1637,7 @@ __global__ void __launch_bounds__(PCG_THREADS, 1) k_pcg(PcgArgs A) {
     done = (s_conv[0] & s_conv[1] & s_conv[2]) != 0;
   }
   trace_mark(A, 3);
-  // ---- FP64 copy of the solution for the spreading; body forces
-  // F_w = -sum_l 2 rho_l w_l (Eq. 26 x ds, Sec. 3.7): block b reduces body b in
-  // a fixed order (lane-strided FP64 sums, fixed shuffle tree, warp order)
+  // ---- FP64 copy of the solution
   for (int i = gtid; i < 3 * m; i += nthreads) A.w[i] = df_to_double(A.wd[i]);
   // every block left the loop after the same barrier: the whole solution is
   // final, so the spreading runs here instead of in a kernel of its own
@@ -1516,38 +1646,444 @@ __global__ void __launch_bounds__(PCG_THREADS, 1) k_pcg(PcgArgs A) {
     for (long long gi = gtid; gi < tot; gi += nthreads)
       spread_node(gi, m, A.base, A.wts, A.wd, A.tile_slot, A.geo, A.acc, A.status);
   }
-  for (int b = blockIdx.x; b < A.nbodies; b += gridDim.x) {
-    double v[3] = {0, 0, 0};
-    for (int l = A.boff[b] + threadIdx.x; l < A.boff[b + 1]; l += blockDim.x)
-      for (int c = 0; c < 3; ++c) {
-        const double f = 2.0 * A.rho_l[l] * df_to_double(A.wd[3 * l + c]);   // force on the fluid
-        A.mforce[3 * l + c] = f;
-        v[c] += f;
+  finish_solve(A, it, done, rebuild, s_scale, s_rz, shd);
+}
+
+// ------------------------------------------------------------------ the solve on one cluster
+// The same conjugate gradients with the dense per-body inverse, for marker sets
+// that one thread-block cluster holds (up to 16 blocks).  What bounds a small solve is latency: in k_pcg an
+// iteration cost 13 us at 68 to 520 markers on 68 to 76 blocks, two grid
+// barriers and six L2 round trips (partials, z, r and A p) around 2 us of
+// arithmetic.  Here every block keeps its rows of the recurrence (and, when
+// they fit, of G and M) in shared memory, holds all of z, r and A p in FP32,
+// and pushes its part of them and its partial sums straight into the other
+// blocks' shared memory before a cluster barrier.  Blocks own contiguous rows.
+//
+// An iteration runs every instruction of its loop once, so instruction fetch
+// counts as much as arithmetic (unrolled and with 1024 threads it took 6 us at
+// 68 markers, a third of the issue slots lost to fetches): the double-float trees
+// are loops, the divisions one function, and a block has 512 threads.
+constexpr int CLUSTER_MAX = 16;
+constexpr int CLUSTER_THREADS = 512;
+constexpr int CLUSTER_WARPS = CLUSTER_THREADS / 32;
+
+
+struct ClusterArgs {
+  int rows;          // rows per block (even)
+  int lanes;         // lanes per preconditioner row pair: 8, 16 or 32
+  int slot;          // floats per resident preconditioner row (0: rows read from L2)
+  int o_xa, o_xr, o_ys, o_meta, o_part, o_m, o_g;   // shared-memory offsets in bytes (z at 0)
+  int g_bytes;       // room for the block's rows of G
+};
+
+// sum_j M_lj x_j of rows l0 and l0 + 1 over a group of `lanes` lanes; x is one
+// padded FP32 vector of all bodies in shared memory, row0 / row1 the rows'
+// FP32 values (shared or global).  Every lane of the group ends with the sums.
+__device__ __forceinline__ void cluster_pair(const float4* __restrict__ row0, const float4* __restrict__ row1, bool in_l2,
+                                             const float* __restrict__ x0, const float* __restrict__ x1, int nq0, int nq1,
+                                             int lanes, int gl, float z0[3], float z1[3]) {
+  float a0 = 0.f, a1 = 0.f, a2 = 0.f, b0 = 0.f, b1 = 0.f, b2 = 0.f;
+  if (x0 == x1) {
+#pragma unroll 2
+    for (int q = gl; q < nq0; q += lanes) {
+      const float4 m0 = in_l2 ? __ldcg(row0 + q) : row0[q];
+      const float4 m1 = in_l2 ? __ldcg(row1 + q) : row1[q];
+      const float4* xv = reinterpret_cast<const float4*>(x0 + 12 * q);
+      const float4 v0 = xv[0], v1 = xv[1], v2 = xv[2];
+      a0 = fmaf(m0.x, v0.x, a0); a1 = fmaf(m0.x, v0.y, a1); a2 = fmaf(m0.x, v0.z, a2);
+      a0 = fmaf(m0.y, v0.w, a0); a1 = fmaf(m0.y, v1.x, a1); a2 = fmaf(m0.y, v1.y, a2);
+      a0 = fmaf(m0.z, v1.z, a0); a1 = fmaf(m0.z, v1.w, a1); a2 = fmaf(m0.z, v2.x, a2);
+      a0 = fmaf(m0.w, v2.y, a0); a1 = fmaf(m0.w, v2.z, a1); a2 = fmaf(m0.w, v2.w, a2);
+      b0 = fmaf(m1.x, v0.x, b0); b1 = fmaf(m1.x, v0.y, b1); b2 = fmaf(m1.x, v0.z, b2);
+      b0 = fmaf(m1.y, v0.w, b0); b1 = fmaf(m1.y, v1.x, b1); b2 = fmaf(m1.y, v1.y, b2);
+      b0 = fmaf(m1.z, v1.z, b0); b1 = fmaf(m1.z, v1.w, b1); b2 = fmaf(m1.z, v2.x, b2);
+      b0 = fmaf(m1.w, v2.y, b0); b1 = fmaf(m1.w, v2.z, b1); b2 = fmaf(m1.w, v2.w, b2);
+    }
+  } else {   // the pair straddles two bodies, or the second row does not exist (nq1 = 0)
+#pragma unroll 1
+    for (int h = 0; h < 2; ++h) {
+      const float4* row = h ? row1 : row0;
+      const float* x = h ? x1 : x0;
+      const int nq = h ? nq1 : nq0;
+      float s0 = 0.f, s1 = 0.f, s2 = 0.f;
+#pragma unroll 1
+      for (int q = gl; q < nq; q += lanes) {
+        const float4 m0 = in_l2 ? __ldcg(row + q) : row[q];
+        const float4* xv = reinterpret_cast<const float4*>(x + 12 * q);
+        const float4 v0 = xv[0], v1 = xv[1], v2 = xv[2];
+        s0 = fmaf(m0.x, v0.x, s0); s1 = fmaf(m0.x, v0.y, s1); s2 = fmaf(m0.x, v0.z, s2);
+        s0 = fmaf(m0.y, v0.w, s0); s1 = fmaf(m0.y, v1.x, s1); s2 = fmaf(m0.y, v1.y, s2);
+        s0 = fmaf(m0.z, v1.z, s0); s1 = fmaf(m0.z, v1.w, s1); s2 = fmaf(m0.z, v2.x, s2);
+        s0 = fmaf(m0.w, v2.y, s0); s1 = fmaf(m0.w, v2.z, s1); s2 = fmaf(m0.w, v2.w, s2);
       }
-    for (int o = 16; o > 0; o >>= 1)
-      for (int c = 0; c < 3; ++c) v[c] += __shfl_xor_sync(0xffffffffu, v[c], o);
-    block_total3(v, shd);
-    if (threadIdx.x == 0) {
-      double* h = A.hist + ((long long)b * HIST_LEN + (A.step % HIST_LEN)) * 3;
-      for (int c = 0; c < 3; ++c) h[c] = -v[c];   // force on the body
+      if (h == 0) { a0 = s0; a1 = s1; a2 = s2; }
+      else { b0 = s0; b1 = s1; b2 = s2; }
     }
   }
-  if (gtid == 0) {
-    double rel = 0.0;
-    for (int c = 0; c < A.D; ++c)
-      if (s_scale[c].hi > 0.f) rel = fmax(rel, sqrt(fmax(df_to_double(s_rz[c]), 0.0) / df_to_double(s_scale[c])));
-    A.info[0] = it;
-    if (rebuild) {
-      A.info[4] = it;
-      A.info[5] = 0;
-    } else {
-      A.info[5] = min(A.info[5] + max(it - max(A.info[4], REBUILD_ITERS_OK), 0), 1 << 30);
-    }
-    A.info[1] = (A.info[5] > A.rebuild_excess || !done) ? 1 : 0;
-    A.info[2] = done ? 1 : 0;
-    *A.res = rel;
-    if (!done) atomicOr(A.status, ST_NOTCONV);
+  __syncwarp();
+#pragma unroll 1
+  for (int o = lanes >> 1; o > 0; o >>= 1) {
+    a0 += __shfl_xor_sync(0xffffffffu, a0, o);
+    a1 += __shfl_xor_sync(0xffffffffu, a1, o);
+    a2 += __shfl_xor_sync(0xffffffffu, a2, o);
+    b0 += __shfl_xor_sync(0xffffffffu, b0, o);
+    b1 += __shfl_xor_sync(0xffffffffu, b1, o);
+    b2 += __shfl_xor_sync(0xffffffffu, b2, o);
   }
+  z0[0] = a0; z0[1] = a1; z0[2] = a2;
+  z1[0] = b0; z1[1] = b1; z1[2] = b2;
+}
+
+// Sums of the owners' contributions per component: every owner warp's total,
+// then, in warp order, component c's total into slot `rank` of every block's
+// part[][3] (warp c, lane k to block k).
+// copy(block) runs between the two, one warp per destination block.
+template <class Copy>
+__device__ __forceinline__ void cluster_push(cg::cluster_group& cl, df v, bool owner_warp, int wpc, df* sh, df* part,
+                                             int cs, int rank, Copy copy) {
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  if (owner_warp) {
+    v = df_warp_sum(v);
+    if (lane == 0) sh[wid] = v;
+  }
+  __syncthreads();
+  if (wid < 3 && lane < cs) {
+    df t = sh[wid * wpc];
+#pragma unroll 1
+    for (int k = 1; k < wpc; ++k) t = df_add(t, sh[wid * wpc + k]);
+    (cs == 1 ? part : cl.map_shared_rank(part, lane))[3 * rank + wid] = t;
+  }
+  if (cs > 1) {
+#pragma unroll 1
+    for (int k = wid; k < cs; k += CLUSTER_WARPS)
+      if (k != rank) copy(k);
+  }
+}
+__device__ __forceinline__ void cluster_barrier(cg::cluster_group& cl, int cs) {
+  if (cs == 1) __syncthreads();
+  else cl.sync();
+}
+// After the cluster barrier: the total of component c over the blocks, in every lane.
+__device__ __forceinline__ df cluster_total(const df* part, int c, int cs) {
+  const int lane = threadIdx.x & 31;
+  if (cs == 1) return part[c];
+  return df_warp_sum(lane < cs ? part[3 * lane + c] : df_make(0.f, 0.f), CLUSTER_MAX);
+}
+
+// Work split within a block: thread c Rp + i (Rp = rows rounded up to warps)
+// owns row i of component c, holds its r, p, A p and w in registers and forms
+// its row of G z alone; the preconditioner's row pairs go to groups of lanes.
+// With eight lanes a row and three components a lane, as in k_pcg, the
+// double-float butterflies and the updates were done by three lanes of eight.
+__global__ void __launch_bounds__(CLUSTER_THREADS, 1) k_pcg_cluster(PcgArgs A, ClusterArgs S) {
+  cg::cluster_group cl = cg::this_cluster();
+  extern __shared__ __align__(16) float sm[];
+  __shared__ double shd[3 * PCG_WARPS + 8];
+  __shared__ df shdf[2][CLUSTER_WARPS];
+  __shared__ df s_rz[3], s_scale[3], s_beta[3], s_alpha[3], s_stop[3];
+  __shared__ float s_alphaf[3];
+  __shared__ int s_conv[3], s_maxnnz;
+  unsigned char* base = reinterpret_cast<unsigned char*>(sm);
+  float* zs = sm;
+  float* xa = reinterpret_cast<float*>(base + S.o_xa);
+  float* xr = reinterpret_cast<float*>(base + S.o_xr);
+  float* ys = reinterpret_cast<float*>(base + S.o_ys);         // M B of the block's rows (set-up)
+  // per row: its slot in the padded vectors, entries of its G row | 128-bit
+  // groups of its M row << 8, its body's slice of the padded vectors, its M row
+  int4* meta = reinterpret_cast<int4*>(base + S.o_meta);
+  df* part = reinterpret_cast<df*>(base + S.o_part);   // [3][CLUSTER_MAX][3]: p.Ap, r.z and, in the set-up, B.MB
+  const int tid = threadIdx.x, lane = tid & 31, wib = tid >> 5;
+  const int cs = gridDim.x, rank = blockIdx.x, m = A.m_total;
+  const int r0 = min(m, rank * S.rows), nr = min(m, r0 + S.rows) - r0;
+  const int rp = (S.rows + 31) & ~31, wpc = rp >> 5;   // owner threads and warps per component
+  const bool owner_warp = tid < 3 * rp;
+  const int oc = owner_warp ? tid / rp : 0, oi = tid - oc * rp;
+  const bool own = owner_warp && oi < nr;
+  const int ol = r0 + (own ? oi : 0);
+  const df dzero = df_make(0.f, 0.f);
+
+  trace_mark(A, 0);
+  const bool rebuild = A.refresh || A.info[1];
+  if (rebuild) {
+    rebuild_dense<CLUSTER_THREADS>(A, cl, sm);
+    __syncthreads();   // the rebuild's shared-memory tiles are reused below
+  }
+  auto token = cl.barrier_arrive();   // no block writes into another before that one has started
+  // ---- this block's rows of M and G
+  if (tid == 0) s_maxnnz = 1;
+  __syncthreads();
+  for (int i = tid; i < S.rows; i += CLUSTER_THREADS) {
+    int4 mt = make_int4(0, 0, -1, 0);
+    if (i < nr) {
+      const int l = r0 + i, bd = A.body_of[l], o = A.boff[bd], ld = precond_ld(A.boff[bd + 1] - o), nnz = A.Gnnz[l];
+      mt = make_int4(A.voff[bd] + 3 * (l - o), nnz | (ld >> 2) << 8, A.voff[bd], (int)A.poff[bd] + (l - o) * ld);
+      atomicMax(&s_maxnnz, nnz);
+    }
+    meta[i] = mt;
+  }
+  // ---- initial guess of all markers (every block forms it from the last solutions)
+  df* w0 = reinterpret_cast<df*>(sm);   // on z and A p, which come later
+  if (A.warm) {
+    for (int i = tid; i < 3 * m; i += CLUSTER_THREADS) {
+      df v = A.wd[i];
+      if (A.warm >= 2) {
+        const df prev = A.wprevd[i];
+        if (A.warm >= 3) {
+          const df t = df_sub(v, prev);
+          v = df_add(df_add(df_add(A.wprev2d[i], t), t), t);
+        } else {
+          v = df_sub(df_make(2.f * v.hi, 2.f * v.lo), prev);
+        }
+      }
+      w0[i] = v;
+    }
+  }
+  __syncthreads();
+  float* mres = reinterpret_cast<float*>(base + S.o_m);
+  if (S.slot > 0) {
+    const int nq = S.slot >> 2;
+#pragma unroll 8
+    for (int e = tid; e < nr * nq; e += CLUSTER_THREADS) {
+      const int i = e / nq, q = e - i * nq;
+      const int4 mt = meta[i];
+      if (q < (mt.y >> 8))
+        reinterpret_cast<float4*>(mres + i * S.slot)[q] = __ldcg(reinterpret_cast<const float4*>(A.M + mt.w) + q);
+    }
+  }
+  const int gstride = s_maxnnz | 1;   // odd: rows start in different banks
+  const bool gres = (long long)nr * gstride * (sizeof(df) + sizeof(unsigned short)) <= (long long)S.g_bytes;
+  df* gv_s = reinterpret_cast<df*>(base + S.o_g);
+  unsigned short* gc_s = reinterpret_cast<unsigned short*>(gv_s + (long long)nr * gstride);
+  if (gres) {
+#pragma unroll 4
+    for (int e = tid; e < nr * gstride; e += CLUSTER_THREADS) {
+      const int i = e / gstride, j = e - i * gstride;
+      if (j < (meta[i].y & 255)) {
+        gv_s[e] = A.Gv[(long long)(r0 + i) * G_MAXNNZ + j];
+        gc_s[e] = (unsigned short)A.Gcol[(long long)(r0 + i) * G_MAXNNZ + j];
+      }
+    }
+  }
+  // zero tails of the padded vectors (never written otherwise)
+  for (int b = 0; b < A.nbodies; ++b) {
+    const int mb = A.boff[b + 1] - A.boff[b], t0 = A.voff[b] + 3 * mb;
+    const int t1 = b + 1 < A.nbodies ? A.voff[b + 1] : A.vtotal;
+    for (int i = t0 + tid; i < t1; i += CLUSTER_THREADS) xr[i] = 0.f;
+  }
+  const df myB = own ? df_from_double(A.B[3 * ol + oc]) : dzero;
+  __syncthreads();
+  cl.barrier_wait(std::move(token));
+  trace_mark(A, 1);
+  // ---- r = B - G w0; r to every block
+  const int4 om = own ? meta[oi] : make_int4(0, 0, 0, 0);
+  const int onnz = om.y & 255, ovi = om.x + oc;
+  const int* gcol = A.Gcol + (long long)ol * G_MAXNNZ;
+  const df* gval = A.Gv + (long long)ol * G_MAXNNZ;
+  df st_r = myB, st_p = dzero, st_ap = dzero, st_w = dzero;
+  if (own) {
+    if (A.warm) {
+      dfacc a0 = acc_zero();
+#pragma unroll 2
+      for (int j = 0; j < onnz; ++j) {
+        const int k = gres ? (int)gc_s[oi * gstride + j] : gcol[j];
+        acc_fma(a0, gres ? gv_s[oi * gstride + j] : gval[j], w0[3 * k + oc]);
+      }
+      st_r = df_sub(myB, acc_value(a0));
+      st_w = w0[3 * ol + oc];
+    }
+    xr[ovi] = st_r.hi;
+  }
+  __syncthreads();
+  // this block's entries of a padded vector to block k, by one warp
+  auto copy_rows = [&](float* x, int k) {
+    float* d = cl.map_shared_rank(x, k);
+#pragma unroll 2
+    for (int e = lane; e < 3 * nr; e += 32) {
+      const int q = meta[e / 3].x + e % 3;
+      d[q] = x[q];
+    }
+  };
+  if (cs > 1) {
+#pragma unroll 1
+    for (int k = wib; k < cs; k += CLUSTER_WARPS)
+      if (k != rank) copy_rows(xr, k);
+  }
+  // ---- B (FP32) in place of A p, for the stopping scale B.(M B)
+  for (int b = 0; b < A.nbodies; ++b) {
+    const int o = A.boff[b], mb = A.boff[b + 1] - o, vo = A.voff[b];
+    const int t1 = (b + 1 < A.nbodies ? A.voff[b + 1] : A.vtotal) - vo;
+    for (int i = tid; i < t1; i += CLUSTER_THREADS) xa[vo + i] = i < 3 * mb ? df_from_double(A.B[3 * o + i]).hi : 0.f;
+  }
+  cluster_barrier(cl, cs);
+  // every block has formed its guess: the last solutions move one back
+  if (A.warm && own) {
+    A.wprev2d[3 * ol + oc] = A.wprevd[3 * ol + oc];
+    A.wprevd[3 * ol + oc] = A.wd[3 * ol + oc];
+  }
+  // ---- row pairs of the preconditioner: a group of S.lanes lanes each; the
+  // products of the block's rows into out[3 i + c]
+  const int lanes = S.lanes, gl = tid & (lanes - 1), grp = tid / lanes, ngrp = CLUSTER_THREADS / lanes;
+  const int npairs = (nr + 1) >> 1;
+  auto precondition = [&](const float* x, float* out) {
+#pragma unroll 1
+    for (int p0 = 0; p0 < npairs; p0 += ngrp) {
+      if (p0 + (tid & ~31) / lanes >= npairs) break;   // no pair left for this warp
+      const bool live = p0 + grp < npairs;
+      const int p = live ? p0 + grp : 0;
+      const int4 m0 = meta[2 * p], m1 = meta[2 * p + 1];   // S.rows is even
+      const float *row0, *row1;
+      if (S.slot > 0) {
+        row0 = mres + 2 * p * S.slot;
+        row1 = row0 + S.slot;
+      } else {
+        row0 = A.M + m0.w;
+        row1 = A.M + m1.w;
+      }
+      float z0[3], z1[3];
+      cluster_pair(reinterpret_cast<const float4*>(row0), reinterpret_cast<const float4*>(row1), S.slot == 0, x + m0.z,
+                   m1.z >= 0 ? x + m1.z : nullptr, m0.y >> 8, m1.y >> 8, lanes, gl, z0, z1);
+      if (live && gl == 0) {
+        float* o = out + 6 * p;
+        o[0] = z0[0];
+        o[1] = z0[1];
+        o[2] = z0[2];
+        if (2 * p + 1 < nr) {
+          o[3] = z1[0];
+          o[4] = z1[1];
+          o[5] = z1[2];
+        }
+      }
+    }
+    __syncthreads();
+  };
+  float* zown = zs + 3 * r0;
+  auto copy_z = [&](int k) {
+    float* d = cl.map_shared_rank(zown, k);
+#pragma unroll 2
+    for (int e = lane; e < 3 * nr; e += 32) d[e] = zown[e];
+  };
+  auto copy_none = [](int) {};
+  precondition(xr, zown);
+  precondition(xa, ys);
+  {
+    df rz = dzero, bb = dzero;
+    if (own) {
+      const float z = zown[3 * oi + oc];
+      rz = df_mul_f(st_r, z);
+      bb = df_mul_f(myB, ys[3 * oi + oc]);
+    }
+    cluster_push(cl, bb, owner_warp, wpc, shdf[0], part + 6 * CLUSTER_MAX, cs, rank, copy_none);
+    cluster_push(cl, rz, owner_warp, wpc, shdf[1], part + 3 * CLUSTER_MAX, cs, rank, copy_z);
+  }
+  cluster_barrier(cl, cs);
+  trace_mark(A, 2);
+  if (wib < 3) {
+    const int c = wib;
+    const df sc = cluster_total(part + 6 * CLUSTER_MAX, c, cs), rz = cluster_total(part + 3 * CLUSTER_MAX, c, cs);
+    if (lane == 0) {
+      s_scale[c] = sc;
+      s_rz[c] = rz;
+      s_beta[c] = dzero;
+      s_stop[c] = df_from_double(A.tol * A.tol * df_to_double(sc));
+      s_conv[c] = (c >= A.D || !df_greater(rz, s_stop[c])) ? 1 : 0;
+    }
+  }
+  __syncthreads();
+  int it = 0;
+  bool done = (s_conv[0] & s_conv[1] & s_conv[2]) != 0;
+  while (!done && it < PCG_MAX_ITERS) {
+    // ---- P1: p = z + beta p;  A p = G z + beta A p;  partial p.Ap;  r and A p (FP32) to every block
+    // (the phases of an iteration are not marked: reading the timer would show in them)
+    trace_mark(A, it < 26 ? 8 + TRACE_PER_IT * it : TRACE_SLOTS);
+    df pAp = dzero;
+    if (own) {
+      dfacc a0 = acc_zero();
+      if (gres) {
+        const unsigned short* gc = gc_s + oi * gstride;
+        const df* gv = gv_s + oi * gstride;
+#pragma unroll 4
+        for (int j = 0; j < onnz; ++j) acc_fma_f(a0, gv[j], zs[3 * (int)gc[j] + oc]);
+      } else {
+#pragma unroll 4
+        for (int j = 0; j < onnz; ++j) acc_fma_f(a0, gval[j], zs[3 * gcol[j] + oc]);
+      }
+      const df beta = s_beta[oc];
+      st_p = df_add(df_from_float(zown[3 * oi + oc]), df_mul(beta, st_p));
+      st_ap = df_add(acc_value(a0), df_mul(beta, st_ap));
+      xa[ovi] = st_ap.hi;
+      xr[ovi] = st_r.hi;
+      pAp = df_mul(st_p, st_ap);
+    }
+    cluster_push(cl, pAp, owner_warp, wpc, shdf[0], part, cs, rank, [&](int k) {
+      copy_rows(xa, k);
+      copy_rows(xr, k);
+    });
+    cluster_barrier(cl, cs);
+    // ---- P2: alpha;  z = M (r - alpha A p) in FP32;  w += alpha p;  r -= alpha A p;  partial r.z
+    if (wib < 3) {
+      const int c = wib;
+      const df tot = cluster_total(part, c, cs);
+      const df a = (tot.hi > 0.f && s_rz[c].hi > 0.f) ? df_div_call(s_rz[c], tot) : dzero;
+      if (lane == 0) {
+        s_alpha[c] = a;
+        s_alphaf[c] = a.hi;
+      }
+    }
+    __syncthreads();
+    for (int q = tid; q < (A.vtotal >> 2); q += CLUSTER_THREADS) {
+      // entry 4 q + k is component (4 q + k) mod 3 (the slices start at multiples of 12)
+      const int c0 = q % 3;   // (4 q) mod 3
+      const float f0 = s_alphaf[c0], f1 = s_alphaf[c0 == 2 ? 0 : c0 + 1], f2 = s_alphaf[c0 == 0 ? 2 : c0 - 1];
+      float4 v = reinterpret_cast<const float4*>(xr)[q];
+      const float4 a = reinterpret_cast<const float4*>(xa)[q];
+      v.x = fmaf(-f0, a.x, v.x);
+      v.y = fmaf(-f1, a.y, v.y);
+      v.z = fmaf(-f2, a.z, v.z);
+      v.w = fmaf(-f0, a.w, v.w);
+      reinterpret_cast<float4*>(xr)[q] = v;
+    }
+    __syncthreads();
+    precondition(xr, zown);
+    df rz = dzero;
+    if (own) {
+      const df alpha = s_alpha[oc];
+      const float z = zown[3 * oi + oc];
+      st_w = df_add(st_w, df_mul(alpha, st_p));
+      st_r = df_sub(st_r, df_mul(alpha, st_ap));
+      rz = df_mul_f(st_r, z);
+    }
+    cluster_push(cl, rz, owner_warp, wpc, shdf[1], part + 3 * CLUSTER_MAX, cs, rank, copy_z);
+    cluster_barrier(cl, cs);
+    if (wib < 3) {
+      const int c = wib;
+      const df rzn = cluster_total(part + 3 * CLUSTER_MAX, c, cs);
+      const df prev = s_rz[c];
+      const df beta = prev.hi > 0.f ? df_div_call(rzn, prev) : dzero;
+      __syncwarp();
+      if (lane == 0) {
+        s_beta[c] = beta;
+        s_rz[c] = rzn;
+        s_conv[c] = (c >= A.D || !df_greater(rzn, s_stop[c])) ? 1 : 0;
+      }
+    }
+    __syncthreads();
+    ++it;
+    done = (s_conv[0] & s_conv[1] & s_conv[2]) != 0;
+  }
+  trace_mark(A, 3);
+  // ---- the solution, the spreading of this block's rows, the body forces
+  if (own) {
+    A.wd[3 * ol + oc] = st_w;
+    A.w[3 * ol + oc] = df_to_double(st_w);
+  }
+  __syncthreads();
+  {
+    const int nn = A.geo.D == 3 ? 64 : 16;
+    for (int e = tid; e < nr * nn; e += CLUSTER_THREADS)
+      spread_node((long long)r0 * nn + e, m, A.base, A.wts, A.wd, A.tile_slot, A.geo, A.acc, A.status);
+  }
+  cluster_barrier(cl, cs);
+  finish_solve(A, it, done, rebuild, s_scale, s_rz, shd);
 }
 
 // ------------------------------------------------------------------ forces
@@ -1637,8 +2173,9 @@ cudaError_t ib_alloc(ibl_ctx* c) {
   IBL_CU(cudaMalloc(&c->d_tile_slot, sizeof(int) * c->tg.n_tiles));
   IBL_CU(cudaMemsetAsync(c->d_tile_slot, 0xff, sizeof(int) * c->tg.n_tiles, c->stream));
   IBL_CU(cudaMalloc(&c->d_slot_tile, sizeof(int) * c->cap_slots));
-  IBL_CU(cudaMalloc(&c->d_band_count, sizeof(int)));
-  IBL_CU(cudaMemsetAsync(c->d_band_count, 0, sizeof(int), c->stream));
+  IBL_CU(cudaMalloc(&c->d_band_count, 2 * sizeof(int)));
+  IBL_CU(cudaMemsetAsync(c->d_band_count, 0, 2 * sizeof(int), c->stream));
+  c->front_parity = 0;
   IBL_CU(cudaMalloc(&c->d_tile_mcount, sizeof(int) * c->cap_slots));
   IBL_CU(cudaMemsetAsync(c->d_tile_mcount, 0, sizeof(int) * c->cap_slots, c->stream));
   IBL_CU(cudaMalloc(&c->d_tile_markers, sizeof(int) * (size_t)c->cap_slots * TILE_MARKER_CAP));
@@ -1916,14 +2453,53 @@ cudaError_t ib_step_front(ibl_ctx* c) {
   }
   const int tb = 64;
   const int mb = (m + tb - 1) / tb;
-  k_kinematics<<<(3 * m + 127) / 128, 128, 0, c->stream>>>(bt, m, c->d_body, c->d_X0, c->d_Xp, c->d_Up, c->d_X, c->d_U,
-                                         c->d_base, reinterpret_cast<df*>(c->d_wts), (double)c->step, g,
-                                         c->d_status);
-  phase_mark(c, 0);
+  MotionArgs M;
+  M.body_of = c->d_body;
+  M.X0 = c->d_X0;
+  M.Xp = c->d_Xp;
+  M.Up = c->d_Up;
+  M.X = c->d_X;
+  M.U = c->d_U;
+  M.base = c->d_base;
+  M.wts = reinterpret_cast<df*>(c->d_wts);
+  M.status = c->d_status;
   // candidate-list assembly unless a body is driven by uploaded states this step
   bool any_prescribed = false;
   for (auto& b : c->bodies) any_prescribed |= b.prescribed;
   const int use_tiles_host = any_prescribed ? 1 : 0;
+  if (m <= FRONT_MARKERS) {
+    FrontArgs F;
+    F.m = m;
+    F.cap = c->cap_slots;
+    F.cur = c->front_parity ^= 1;
+    F.use_tiles = use_tiles_host;
+    F.tile_slot = c->d_tile_slot;
+    F.slot_tile = c->d_slot_tile;
+    F.counts = c->d_band_count;
+    F.tile_mcount = c->d_tile_mcount;
+    F.tile_markers = c->d_tile_markers;
+    F.mixed = c->d_mixed;
+    F.rowsum_max = c->d_Gdiag_max;
+    // one block up to 128 markers; eight above, for their FP64 units
+    const int blocks = m <= 128 ? 1 : 8, threads = m <= 512 ? 256 : 512;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(blocks);
+    cfg.blockDim = dim3(threads);
+    cfg.stream = c->stream;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = blocks;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    IBL_CU(cudaLaunchKernelEx(&cfg, c->prec == IBL_FP64 ? k_ib_front<true> : k_ib_front<false>, bt, M, g, F));
+    for (int ph = 0; ph < 4; ++ph) phase_mark(c, ph);
+    c->launches++;
+    return cudaGetLastError();
+  }
+  if (c->prec == IBL_FP64) k_kinematics<true><<<(m + 31) / 32, 32, 0, c->stream>>>(bt, m, M, g);
+  else k_kinematics<false><<<(m + 31) / 32, 32, 0, c->stream>>>(bt, m, M, g);
+  phase_mark(c, 0);
   IBL_CU(cudaMemsetAsync(c->d_mixed, use_tiles_host, sizeof(int), c->stream));
   IBL_CU(cudaMemsetAsync(c->d_band_count, 0, sizeof(int), c->stream));
   phase_mark(c, 1);
@@ -1937,21 +2513,84 @@ cudaError_t ib_step_front(ibl_ctx* c) {
   return cudaGetLastError();
 }
 
+// The solve on one cluster: for marker sets up to CLUSTER_MARKERS, with the
+// automatic preconditioner (an explicit kind or streamed rows keep k_pcg, whose
+// block count the caller may then choose).  One block per CLUSTER_ROWS rows,
+// 1 to 16.
+// G and M stay in shared memory when they fit, else they are read from L2.
+constexpr int CLUSTER_ROWS = 72;
+static bool cluster_plan(const ibl_ctx* c, const PcgArgs& A, ClusterArgs& S, int& blocks, size_t& smem) {
+  const int m = c->m_total;
+  if (c->sep_on || c->precond_kind != -1 || c->resident_rows != -1 || m > CLUSTER_MARKERS) return false;
+  blocks = 1;
+  while (blocks < CLUSTER_MAX && blocks * CLUSTER_ROWS < m) blocks *= 2;
+  const int rows = (m + blocks - 1) / blocks;
+  S.rows = (rows + 1) & ~1;
+  S.lanes = 32;
+  while (S.lanes > 8 && (S.rows / 2) * S.lanes > CLUSTER_THREADS) S.lanes /= 2;
+  const auto up = [](size_t b) { return (b + 15) & ~(size_t)15; };
+  size_t o = up(sizeof(float) * 3 * (size_t)m);
+  S.o_xa = (int)o;
+  o = std::max(o + up(sizeof(float) * (size_t)A.vtotal), up(sizeof(df) * 3 * (size_t)m));   // w0 lies on z and A p
+  S.o_xr = (int)o;
+  o += up(sizeof(float) * (size_t)A.vtotal);
+  S.o_ys = (int)o;
+  o += up(sizeof(float) * 3 * (size_t)S.rows);
+  S.o_meta = (int)o;
+  o += sizeof(int4) * (size_t)S.rows;
+  S.o_part = (int)o;
+  o += up(sizeof(df) * 9 * CLUSTER_MAX);
+  int slot = 0;
+  for (auto& b : c->bodies) slot = std::max(slot, precond_ld(b.m));
+  const size_t mrows = sizeof(float) * (size_t)S.rows * slot;
+  S.o_m = (int)o;
+  S.slot = o + mrows <= PCG_SMEM_MAX ? slot : 0;
+  if (S.slot) o += up(mrows);
+  S.o_g = (int)o;
+  if (o > PCG_SMEM_MAX) return false;
+  // room for rows of up to 64 entries (a unit-spaced sheet has 49)
+  const size_t g = std::min(up((size_t)S.rows * 64 * (sizeof(df) + sizeof(unsigned short))), PCG_SMEM_MAX - o);
+  S.g_bytes = (int)g;
+  smem = std::max(o + g, GJ_SMEM);
+  return true;
+}
+
+static cudaError_t launch_cluster(ibl_ctx* c, PcgArgs& A, ClusterArgs& S, int blocks, size_t smem) {
+  static bool attr_set = false;
+  if (!attr_set) {
+    IBL_CU(cudaFuncSetAttribute((const void*)k_pcg_cluster, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PCG_SMEM_MAX));
+    IBL_CU(cudaFuncSetAttribute((const void*)k_pcg_cluster, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+    attr_set = true;
+  }
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(blocks);
+  cfg.blockDim = dim3(CLUSTER_THREADS);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = c->stream;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = blocks;
+  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, k_pcg_cluster, A, S);
+}
+
 // Marker lists, interpolation, assembly, the implicit solve and spreading.
 cudaError_t ib_step_back(ibl_ctx* c) {
   const int m = c->m_total;
   if (m == 0) return cudaSuccess;
   Geo g = make_geo(c);
-  const int tb = 64;
-  const int mb = (m + tb - 1) / tb;
-  k_append_markers<<<(8 * m + 255) / 256, 256, 0, c->stream>>>(m, c->d_base, g, c->d_tile_slot, c->d_tile_mcount,
-                                             c->d_tile_markers, c->d_status, c->d_body, c->d_slot_body,
-                                             c->d_mixed);
+  if (m > FRONT_MARKERS) {
+    k_append_markers<<<(8 * m + 255) / 256, 256, 0, c->stream>>>(m, c->d_base, g, c->d_tile_slot, c->d_tile_mcount,
+                                                                 c->d_tile_markers, c->d_status, c->d_body,
+                                                                 c->d_slot_body, c->d_mixed);
+    c->launches += 1;
+    IBL_CU(cudaGetLastError());
+    IBL_CU(cudaMemsetAsync(c->d_Gdiag_max, 0, sizeof(double) * MAX_BODIES, c->stream));
+  }
   phase_mark(c, 4);
   for (auto& b : c->bodies) b.prescribed = false;
-  c->launches += 1;
-  IBL_CU(cudaGetLastError());
-  IBL_CU(cudaMemsetAsync(c->d_Gdiag_max, 0, sizeof(double) * MAX_BODIES, c->stream));
   IBL_CU(interpolate(c, g));   // interpolation and assembly, one launch
   phase_mark(c, 5);
   phase_mark(c, 6);
@@ -2041,14 +2680,21 @@ cudaError_t ib_step_back(ibl_ctx* c) {
   A.sep = c->d_sep;
   A.sep_on = c->sep_on ? 1 : 0;
   if (c->sep_on && A.refresh) IBL_CU(sep_launch(c, g.n, g.per));
-  static bool smem_set = false;
-  if (!smem_set) {
-    IBL_CU(cudaFuncSetAttribute((const void*)k_pcg, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PCG_SMEM_MAX));
-    smem_set = true;
+  ClusterArgs S;
+  int cluster = 0;
+  size_t cluster_smem = 0;
+  if (cluster_plan(c, A, S, cluster, cluster_smem)) {
+    IBL_CU(launch_cluster(c, A, S, cluster, cluster_smem));
+  } else {
+    static bool smem_set = false;
+    if (!smem_set) {
+      IBL_CU(cudaFuncSetAttribute((const void*)k_pcg, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PCG_SMEM_MAX));
+      smem_set = true;
+    }
+    void* args[] = {&A};
+    IBL_CU(cudaLaunchCooperativeKernel((void*)k_pcg, dim3(pcg_blocks), dim3(PCG_THREADS), args, c->pcg_smem,
+                                       c->stream));
   }
-  void* args[] = {&A};
-  IBL_CU(cudaLaunchCooperativeKernel((void*)k_pcg, dim3(pcg_blocks), dim3(PCG_THREADS), args, c->pcg_smem,
-                                     c->stream));
   phase_mark(c, 7);
   c->launches++;
   c->warm = true;

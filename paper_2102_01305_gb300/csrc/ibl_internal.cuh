@@ -78,6 +78,7 @@ struct ibl_ctx {
   cudaEvent_t ev_bulk = nullptr;    // bulk collide done (stream_bulk)
   int overlap = -1;                 // -1 automatic, 0 off, 1 on
   int collide_bx = 64, collide_by = 2;   // thread block of the one-kernel collide
+  bool collide_auto = true;              // not set by the caller: see cell_block (lbm.cu)
   int collide_pairs = 3;             // 16-bit storage: 3 two cells and ZP planes per thread, 1 two cells,
                                      // 2 staged planes, 0 one cell per thread
   size_t elem = 4;               // bytes per stored population
@@ -122,7 +123,8 @@ struct ibl_ctx {
   ibl::BodyDev* d_bodies = nullptr;
   int* d_tile_slot = nullptr;    // n_tiles
   int* d_slot_tile = nullptr;    // cap_slots
-  int* d_band_count = nullptr;   // 1 int: used slots
+  int* d_band_count = nullptr;   // used slots: [front_parity]; the other one is the last step's on one cluster
+  int front_parity = 0;          // flips each step when the front runs on one cluster, else 0
   int* d_tile_mcount = nullptr;  // cap_slots
   int* d_tile_markers = nullptr; // cap_slots x TILE_MARKER_CAP
   void* d_band_F = nullptr;      // cap_slots x 3 x TILE_CELLS (real)
@@ -245,6 +247,10 @@ int pcg_block_count(const ibl_ctx* c);
 // solve (dense per-body preconditioner, m^2 per iteration) dominates and
 // gets every SM.
 constexpr int SPLIT_MAX_MARKERS = 8192;
+// Cells from which the step is split: 96^3 with 2 x 260 markers takes 137 us a
+// step split and 148 unsplit, 800 x 400 with 2 x 34 markers 105 and 107, 200 x 100
+// 75 and 70.
+constexpr long long SPLIT_MIN_CELLS = 1LL << 18;
 cudaError_t launch_force_field(ibl_ctx* c, double* d_out);
 
 // separable preconditioner (sep.cu)

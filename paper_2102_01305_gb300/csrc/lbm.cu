@@ -499,6 +499,10 @@ __global__ void __launch_bounds__(256, IB ? 3 : IBL_PAIRS_MIN_BLOCKS) k_collide_
 #define IBL_ZP 8
 #endif
 constexpr int ZP = IBL_ZP;   // planes per thread
+// Fewest threads for which it pays: 64^3 (32768) takes 10.4 us a step against
+// 7.2 with one plane a thread, 96^3 (73728) 18.5 against 17.2, 128^3 (131072)
+// 34.5 against 35.0.
+constexpr long long ZP_MIN_THREADS = 131072;
 
 template <int Q, class T>
 struct PairWords {
@@ -1058,8 +1062,16 @@ FluidParams<R> make_params(ibl_ctx* c, bool with_ib) {
   return p;
 }
 
-static dim3 cell_block(ibl_ctx* c) {
-  return dim3(c->collide_bx, c->collide_by, 1);
+// Thread block for rows of n threads: the caller's, or 64 x 2, or 32 x 4 where
+// 32 leaves fewer lanes idle at the row's end (192^3 in 16 bits, 96 threads a
+// row: 99 us a step against 111).
+// Grids of few cells take one warp a block, so that the last block of an SM
+// is a small one (200 x 100 cells in FP64: 131 cells an SM on average, 256 with
+// 128-thread blocks).
+static dim3 cell_block(ibl_ctx* c, int n) {
+  if (!c->collide_auto) return dim3(c->collide_bx, c->collide_by, 1);
+  if (c->N < 512LL * num_sms()) return dim3(32, 1, 1);
+  return (n + 63) / 64 * 64 > (n + 31) / 32 * 32 ? dim3(32, 4, 1) : dim3(64, 2, 1);
 }
 static dim3 cell_grid(ibl_ctx* c, dim3 b) {
   return dim3((c->nx + b.x - 1) / b.x, (c->ny + b.y - 1) / b.y, c->nz);
@@ -1084,7 +1096,8 @@ cudaError_t collide_fg(ibl_ctx* c, bool with_ib) {
   using R = typename Store<T>::R;
   auto p = make_params<R>(c, with_ib);
   const DirPtrs<Q, T> P = dir_ptrs<Q, T>(c);
-  dim3 b = cell_block(c), g = cell_grid(c, b);
+  dim3 b = cell_block(c, sizeof(T) == 2 && !c->poststream && c->nx % 2 == 0 && c->collide_pairs ? c->nx / 2 : c->nx);
+  dim3 g = cell_grid(c, b);
   if constexpr (sizeof(T) == 2) {
     if constexpr (Q == 19) {
       if (!c->poststream && c->nx % 8 == 0 && c->collide_pairs == 2) {
@@ -1098,10 +1111,13 @@ cudaError_t collide_fg(ibl_ctx* c, bool with_ib) {
         return cudaGetLastError();
       }
     }
-    if (!c->poststream && c->nx % 2 == 0 && c->collide_pairs == 3) {
+    const dim3 zb(b.x, b.y, 1);
+    const dim3 zg((c->nx / 2 + zb.x - 1) / zb.x, (c->ny + zb.y - 1) / zb.y, (c->nz + ZP - 1) / ZP);
+    // below ZP_MIN_THREADS the walking threads are too few to keep the SMs busy,
+    // and one plane a thread is faster
+    const bool few = c->collide_auto && (long long)zg.x * zg.y * zg.z * zb.x * zb.y < ZP_MIN_THREADS;
+    if (!c->poststream && c->nx % 2 == 0 && c->collide_pairs == 3 && !few) {
       // 16-bit storage: two cells per thread, ZP planes per thread
-      const dim3 zb(b.x, b.y, 1);
-      const dim3 zg((c->nx / 2 + zb.x - 1) / zb.x, (c->ny + zb.y - 1) / zb.y, (c->nz + ZP - 1) / ZP);
       if (with_ib) k_collide_pairs_zp<Q, T, true, FG><<<zg, zb, 0, c->stream>>>(P, p);
       else k_collide_pairs_zp<Q, T, false, FG><<<zg, zb, 0, c->stream>>>(P, p);
       c->launches++;
@@ -1149,7 +1165,7 @@ cudaError_t collide_band_q(ibl_ctx* c, int blocks) {
   auto p = make_params<R>(c, true);
   const DirPtrs<Q, T> P = dir_ptrs<Q, T>(c);
   auto kernel = c->poststream ? k_collide_band<Q, T, false> : k_collide_band<Q, T, true>;
-  kernel<<<blocks, TILE_CELLS, 0, c->stream>>>(P, p, c->d_slot_tile, c->d_band_count, c->cap_slots);
+  kernel<<<blocks, TILE_CELLS, 0, c->stream>>>(P, p, c->d_slot_tile, c->d_band_count + c->front_parity, c->cap_slots);
   c->launches++;
   return cudaGetLastError();
 }

@@ -359,7 +359,9 @@ static __device__ void sep_schur(const SepBody* sb, int nb, float* sm, int smem_
         }
         }
       }
-      const df u0 = df_warp_sum(acc_value(a0)), u1 = df_warp_sum(acc_value(a1)), u2 = df_warp_sum(acc_value(a2));
+      df us[3] = {acc_value(a0), acc_value(a1), acc_value(a2)};
+      df_warp_sums(us);
+      const df u0 = us[0], u1 = us[1], u2 = us[2];
       if (lane == 0) {
         B.U[p] = u0.hi + u0.lo;
         B.U[nc + p] = u1.hi + u1.lo;
