@@ -4,7 +4,10 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <mutex>
 #include <string>
+#include <thread>
+#include <vector>
 
 #include "ibl_internal.cuh"
 
@@ -69,6 +72,160 @@ ibl_status ibl::sync_and_collect(ibl_ctx* c) {
 
 static bool is_zh(int b) { return b == IBL_VEL_INLET || b == IBL_PRESS_OUTLET; }
 
+// Device scratch of one set-up or read-out call: the population buffer that
+// the next step will write (its content is dead between steps) when it is large
+// enough, else an allocation.  A cudaMalloc / cudaFree pair of a field waits for
+// the device and maps and unmaps its memory on every call.
+struct Scratch {
+  ibl_ctx* c;
+  double* p = nullptr;
+  bool owned = false;
+  explicit Scratch(ibl_ctx* ctx) : c(ctx) {}
+  cudaError_t get(size_t bytes) {
+    if (bytes <= (size_t)c->Q * (size_t)c->N * c->elem) {
+      p = static_cast<double*>(c->f[c->cur ^ 1]);
+      return cudaSuccess;
+    }
+    owned = true;
+    return cudaMalloc(&p, bytes);
+  }
+  ~Scratch() {
+    if (owned && p) cudaFree(p);
+  }
+};
+
+// ---------------------------------------------------------------- large host transfers
+// A field's copy from or to the caller's pageable memory.  Handed to the driver
+// as a whole, the GPU walks the process's own page tables: 2 ms for 403 MB on
+// untouched tables, but 40 to 130 ms once the kernel's NUMA balancing has
+// unmapped the pages for its sampling (any buffer older than a second), and 15
+// ms of page faults into fresh memory.  So transfers from XFER_MIN bytes go
+// through pinned buffers, several threads copying their own chunks (256^3: u up
+// 4 ms, u and rho down 10; below 64 MB starting the threads costs more than it
+// saves).  The buffers (16 MB a set) are shared by the process's contexts, at
+// most XFER_SETS sets wait for use, and the last context frees them.
+namespace {
+constexpr size_t XFER_MIN = (size_t)64 << 20;
+constexpr size_t XFER_CHUNK = (size_t)1 << 20;
+constexpr int XFER_THREADS = 8;
+constexpr int XFER_SETS = 2;
+
+struct XferSet {
+  char* pin = nullptr;                       // 2 chunks per thread
+  cudaEvent_t ev[2 * XFER_THREADS] = {};
+  int device = 0;
+};
+
+std::mutex g_xfer_mutex;
+std::vector<XferSet> g_xfer_free;
+int g_contexts = 0;
+
+void xfer_free(XferSet& s) {
+  if (s.pin) cudaFreeHost(s.pin);
+  for (auto& e : s.ev)
+    if (e) cudaEventDestroy(e);
+  s = XferSet();
+}
+
+bool xfer_take(int device, XferSet& s) {
+  {
+    std::lock_guard<std::mutex> lock(g_xfer_mutex);
+    for (size_t i = 0; i < g_xfer_free.size(); ++i)
+      if (g_xfer_free[i].device == device) {
+        s = g_xfer_free[i];
+        g_xfer_free.erase(g_xfer_free.begin() + i);
+        return true;
+      }
+  }
+  s.device = device;
+  bool ok = cudaMallocHost(&s.pin, 2 * XFER_THREADS * XFER_CHUNK) == cudaSuccess;
+  for (auto& e : s.ev) ok = ok && cudaEventCreateWithFlags(&e, cudaEventDisableTiming) == cudaSuccess;
+  if (!ok) {
+    cudaGetLastError();
+    xfer_free(s);
+  }
+  return ok;
+}
+
+void xfer_give(XferSet& s) {
+  {
+    std::lock_guard<std::mutex> lock(g_xfer_mutex);
+    if (g_contexts > 0 && (int)g_xfer_free.size() < XFER_SETS) {
+      g_xfer_free.push_back(s);
+      return;
+    }
+  }
+  xfer_free(s);
+}
+
+// One thread's chunks, alternating between its two pinned buffers.
+cudaError_t xfer_chunks(const XferSet& s, int t, int threads, cudaStream_t st, char* dev, char* host, size_t bytes,
+                        bool up) {
+  const size_t n = (bytes + XFER_CHUNK - 1) / XFER_CHUNK;
+  size_t pending[2] = {0, 0};   // chunk + 1 in flight from or to each buffer
+  cudaError_t e = cudaSetDevice(s.device);
+  auto drain = [&](int k) {
+    if (!pending[k]) return;
+    const size_t c = pending[k] - 1;
+    pending[k] = 0;
+    const cudaError_t w = cudaEventSynchronize(s.ev[2 * t + k]);
+    if (e == cudaSuccess) e = w;
+    if (e == cudaSuccess && !up)
+      std::memcpy(host + c * XFER_CHUNK, s.pin + (2 * t + k) * XFER_CHUNK, std::min(XFER_CHUNK, bytes - c * XFER_CHUNK));
+  };
+  int k = 0;
+  for (size_t c = (size_t)t; c < n && e == cudaSuccess; c += (size_t)threads, k ^= 1) {
+    drain(k);
+    if (e != cudaSuccess) break;
+    char* pin = s.pin + (2 * t + k) * XFER_CHUNK;
+    const size_t off = c * XFER_CHUNK, len = std::min(XFER_CHUNK, bytes - off);
+    if (up) {
+      std::memcpy(pin, host + off, len);
+      e = cudaMemcpyAsync(dev + off, pin, len, cudaMemcpyHostToDevice, st);
+    } else {
+      e = cudaMemcpyAsync(pin, dev + off, len, cudaMemcpyDeviceToHost, st);
+    }
+    if (e == cudaSuccess) e = cudaEventRecord(s.ev[2 * t + k], st);
+    if (e == cudaSuccess) pending[k] = c + 1;
+  }
+  drain(k);
+  drain(k ^ 1);
+  return e;
+}
+
+// Copy between device and host memory, ordered on the context's stream; large
+// ones have landed on return, small ones like cudaMemcpyAsync.
+cudaError_t host_copy(ibl_ctx* c, void* dev, void* host, size_t bytes, bool up) {
+  XferSet s;
+  if (bytes < XFER_MIN || !xfer_take(c->device, s))
+    return up ? cudaMemcpyAsync(dev, host, bytes, cudaMemcpyHostToDevice, c->stream)
+              : cudaMemcpyAsync(host, dev, bytes, cudaMemcpyDeviceToHost, c->stream);
+  const int threads = std::max(1, std::min(XFER_THREADS, (int)std::thread::hardware_concurrency() / 2));
+  cudaError_t err[XFER_THREADS];
+  std::vector<std::thread> pool;
+  int started = 0;
+  auto job = [&](int t) {
+    err[t] = xfer_chunks(s, t, threads, c->stream, static_cast<char*>(dev), static_cast<char*>(host), bytes, up);
+  };
+  try {
+    pool.reserve(threads);
+    for (int t = 1; t < threads; ++t) {
+      pool.emplace_back(job, t);
+      started = t;
+    }
+  } catch (...) {   // no thread to be had: its chunks are copied here
+  }
+  job(0);
+  for (int t = started + 1; t < threads; ++t) job(t);
+  for (auto& p : pool) p.join();
+  cudaError_t e = cudaSuccess;
+  for (int t = 0; t < threads; ++t)
+    if (e == cudaSuccess) e = err[t];
+  xfer_give(s);
+  return e;
+}
+}  // namespace
+
 extern "C" {
 
 ibl_status ibl_create(const ibl_grid* grid, double tau, int32_t lattice, ibl_ctx** out) {
@@ -101,6 +258,10 @@ ibl_status ibl_create(const ibl_grid* grid, double tau, int32_t lattice, ibl_ctx
       if (b != zh_axis && bc[2 * b] != IBL_PERIODIC)
         return fail(nullptr, IBL_EINVAL, "a Zou-He face needs periodic lateral axes");
   ibl_ctx* c = new ibl_ctx();
+  {
+    std::lock_guard<std::mutex> lock(g_xfer_mutex);
+    ++g_contexts;
+  }
   c->Q = lattice;
   c->D = D;
   c->nx = grid->nx; c->ny = grid->ny; c->nz = grid->nz;
@@ -164,29 +325,34 @@ ibl_status ibl_destroy(ibl_ctx* c) {
   for (auto& ev : c->pev_pool) cudaEventDestroy(ev);
   if (c->h_stage) cudaFreeHost(c->h_stage);
   if (c->stream) cudaStreamDestroy(c->stream);
+  std::vector<XferSet> unused;
+  {
+    std::lock_guard<std::mutex> lock(g_xfer_mutex);
+    if (--g_contexts == 0) unused.swap(g_xfer_free);
+  }
+  for (auto& s : unused) xfer_free(s);
   delete c;
   return IBL_OK;
 }
 
 ibl_status ibl_init_fluid(ibl_ctx* c, const double* rho, const double* u) {
   if (!c) return IBL_EINVAL;
-  double* d = nullptr;
+  Scratch sc(c);
   const size_t n1 = (size_t)c->N;
   const size_t tot = (rho ? n1 : 0) + (u ? n1 * c->D : 0);
-  if (tot) CK(cudaMalloc(&d, sizeof(double) * tot), "init_fluid alloc");
+  if (tot) CK(sc.get(sizeof(double) * tot), "init_fluid alloc");
+  double* d = sc.p;
   double* d_rho = rho ? d : nullptr;
   double* d_u = u ? d + (rho ? n1 : 0) : nullptr;
   ibl_status st = IBL_OK;
   cudaError_t e = cudaSuccess;
-  if (rho) e = cudaMemcpyAsync(d_rho, rho, sizeof(double) * n1, cudaMemcpyHostToDevice, c->stream);
-  if (e == cudaSuccess && u)
-    e = cudaMemcpyAsync(d_u, u, sizeof(double) * n1 * c->D, cudaMemcpyHostToDevice, c->stream);
+  if (rho) e = host_copy(c, d_rho, const_cast<double*>(rho), sizeof(double) * n1, true);
+  if (e == cudaSuccess && u) e = host_copy(c, d_u, const_cast<double*>(u), sizeof(double) * n1 * c->D, true);
   if (e == cudaSuccess) e = launch_init_eq(c, d_rho, d_u);
   c->poststream = true;
   if (e == cudaSuccess) e = launch_mass_check(c, 0);   // reference total of the mass check
   if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
   st = cuda_check(c, e, "init_fluid");
-  if (d) cudaFree(d);
   if (st != IBL_OK) return st;
   c->initialised = true;
   c->poststream = true;
@@ -198,15 +364,15 @@ ibl_status ibl_init_fluid(ibl_ctx* c, const double* rho, const double* u) {
 
 ibl_status ibl_set_populations(ibl_ctx* c, const double* f) {
   if (!c || !f) return c ? fail(c, IBL_EINVAL, "f is NULL") : IBL_EINVAL;
-  double* d = nullptr;
+  Scratch sc(c);
   const size_t n = (size_t)c->N * c->Q;
-  CK(cudaMalloc(&d, sizeof(double) * n), "set_populations alloc");
-  cudaError_t e = cudaMemcpyAsync(d, f, sizeof(double) * n, cudaMemcpyHostToDevice, c->stream);
+  CK(sc.get(sizeof(double) * n), "set_populations alloc");
+  double* d = sc.p;
+  cudaError_t e = host_copy(c, d, const_cast<double*>(f), sizeof(double) * n, true);
   if (e == cudaSuccess) e = launch_set_pop(c, d);
   c->poststream = true;
   if (e == cudaSuccess) e = launch_mass_check(c, 0);   // reference total of the mass check
   if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
-  cudaFree(d);
   ibl_status st = cuda_check(c, e, "set_populations");
   if (st != IBL_OK) return st;
   c->initialised = true;
@@ -532,14 +698,15 @@ ibl_status ibl_force_history(ibl_ctx* c, int32_t body_id, int64_t max, double* o
   long long avail = std::min<long long>(c->step, HIST_LEN);
   if (!c->ib_ready) avail = 0;
   const long long cnt = std::min<long long>(avail, max);
-  std::vector<double> F(3 * (size_t)HIST_LEN);
-  if (cnt > 0)
-    CK(to_host(c, F.data(), c->d_hist + (size_t)body_id * HIST_LEN * 3, sizeof(double) * 3 * HIST_LEN),
-       "history read");
+  // the asked entries of the ring, in at most two pieces
+  const double* ring = c->d_hist + (size_t)body_id * HIST_LEN * 3;
+  const long long first = (c->step - cnt) % HIST_LEN, head = std::min<long long>(cnt, HIST_LEN - first);
+  if (cnt > 0) CK(to_host(c, out3, ring + 3 * first, sizeof(double) * 3 * head), "history read");
+  if (cnt > head) CK(to_host(c, out3 + 3 * head, ring, sizeof(double) * 3 * (cnt - head)), "history read");
   for (long long k = 0; k < cnt; ++k) {
-    const long long stepk = c->step - cnt + k;
-    const double* f = F.data() + 3 * (stepk % HIST_LEN);
-    coefficients(c, body_id, f, out3 + 3 * k, out3 + 3 * k + 1, out3 + 3 * k + 2);
+    double* o = out3 + 3 * k;
+    const double f[3] = {o[0], o[1], o[2]};
+    coefficients(c, body_id, f, o, o + 1, o + 2);
   }
   if (n) *n = cnt;
   return s;
@@ -553,8 +720,9 @@ ibl_status ibl_get_field(ibl_ctx* c, int32_t what, double* out) {
   ibl_status s = sync_and_collect(c);
   if (s != IBL_OK && s != IBL_ENOTCONV) return s;
   const size_t n = (size_t)c->N * (what == IBL_FIELD_RHO ? 1 : c->D);
-  double* d = nullptr;
-  CK(cudaMalloc(&d, sizeof(double) * n), "field alloc");
+  Scratch sc(c);
+  CK(sc.get(sizeof(double) * n), "field alloc");
+  double* d = sc.p;
   cudaError_t e;
   if (what == IBL_FIELD_FORCE) {
     if (c->m_total == 0 || !c->ib_ready) e = cudaMemsetAsync(d, 0, sizeof(double) * n, c->stream);
@@ -562,9 +730,8 @@ ibl_status ibl_get_field(ibl_ctx* c, int32_t what, double* out) {
   } else {
     e = launch_fields(c, what == IBL_FIELD_RHO ? d : nullptr, what == IBL_FIELD_U ? d : nullptr, nullptr);
   }
-  if (e == cudaSuccess) e = cudaMemcpyAsync(out, d, sizeof(double) * n, cudaMemcpyDeviceToHost, c->stream);
+  if (e == cudaSuccess) e = host_copy(c, d, out, sizeof(double) * n, false);
   if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
-  cudaFree(d);
   CK(e, "get_field");
   return s;
 }
@@ -576,12 +743,12 @@ ibl_status ibl_get_populations(ibl_ctx* c, double* f) {
   ibl_status s = sync_and_collect(c);
   if (s != IBL_OK && s != IBL_ENOTCONV) return s;
   const size_t n = (size_t)c->N * c->Q;
-  double* d = nullptr;
-  CK(cudaMalloc(&d, sizeof(double) * n), "population alloc");
+  Scratch sc(c);
+  CK(sc.get(sizeof(double) * n), "population alloc");
+  double* d = sc.p;
   cudaError_t e = launch_fields(c, nullptr, nullptr, d);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(f, d, sizeof(double) * n, cudaMemcpyDeviceToHost, c->stream);
+  if (e == cudaSuccess) e = host_copy(c, d, f, sizeof(double) * n, false);
   if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
-  cudaFree(d);
   CK(e, "get_populations");
   return s;
 }

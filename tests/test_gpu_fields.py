@@ -79,3 +79,33 @@ def test_collision_with_and_without_force(ibl, prec, force):
     # five steps: the storage's rounding of deviations up to 0.03, a few times per step
     tol = {"fp64": 1e-13, "fp32": 5e-6, "fp16dev": 2e-2}[prec]
     assert rel_err(ctx.ibl_get_field(ibl.IBL_FIELD_U), sim.fields()[1]) < tol
+
+
+# 19 FP64 populations: just under 64 MB (one copy), just over, a ragged last chunk
+@pytest.mark.parametrize("shape", [(76, 76, 76), (76, 76, 77), (79, 81, 83)])
+def test_large_host_transfers_round_trip(ibl, shape):
+    """Exact round trip, four contexts' transfers at once from as many threads."""
+    from concurrent.futures import ThreadPoolExecutor
+    lat = get_lattice(19)
+    rng = np.random.default_rng(6)
+    f = lat.w[:, None, None, None] * (1 + 2.0 ** -20 * rng.integers(-9999, 9999, size=(19,) + shape))
+    g = np.float64(f - lat.w[:, None, None, None]) + lat.w[:, None, None, None]   # what FP64 storage holds
+
+    def trip(k):
+        ctx = _ctx(ibl, 19, shape, "fp64")
+        ctx.ibl_set_populations(np.roll(f, k, axis=1))
+        out = ctx.ibl_get_populations()
+        return np.array_equal(out[gpu_to_oracle_order(ibl, 19)], np.roll(g, k, axis=1)[gpu_to_oracle_order(ibl, 19)])
+
+    with ThreadPoolExecutor(4) as ex:
+        assert all(ex.map(trip, range(4)))
+
+
+def test_force_history_ring(ibl):
+    """The asked number of most recent steps, fewer than, as many as and more than there are."""
+    cfg = W.cylinder_channel(nx=64, ny=40, diameter=10.0, center=(20.0, 20.0), m=31)
+    ctx = ibl.from_workload(cfg)
+    ctx.ibl_step(9)
+    whole = ctx.ibl_force_history(0, 9)
+    assert len(whole) == 9 and np.array_equal(ctx.ibl_force_history(0, 100), whole)
+    assert np.array_equal(ctx.ibl_force_history(0, 4), whole[5:]) and len(ctx.ibl_force_history(0, 0)) == 0
