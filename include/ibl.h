@@ -355,7 +355,8 @@ ibl_status ibl_set_collide_shape(ibl_ctx* ctx, int32_t bx, int32_t by, int32_t p
  * input staged, preconditioner rows done, grid barrier passed.  With the
  * separable preconditioner, [4]-[7] and [251]-[252] mark the ends of stages
  * A-F of the set-up's first application (from [250]) and [253] the end of
- * its stage G.  Unused slots are 0.  Copies min(max, 256) values into ns. */
+ * its stage G.  The solve on one cluster (see ibl_solver_preconditioner) marks
+ * only the first of an iteration's slots.  Unused slots are 0.  Copies min(max, 256) values into ns. */
 ibl_status ibl_solver_trace(ibl_ctx* ctx, int64_t* ns, int32_t max, int32_t* n);
 
 /* Enable (1 or 2) or disable (0) CUDA-event timing of the collide-stream
@@ -369,7 +370,8 @@ ibl_status ibl_profile(ibl_ctx* ctx, int32_t enable);
 /* With ibl_profile(ctx, 2): milliseconds per phase of the step on the
  * context's main stream since profiling was enabled, ms[0..n): 0 kinematics,
  * 1 band counters reset, 2 tile marking, 3 slot assignment (which also
- * resets the previous band), 4 marker lists,
+ * resets the previous band), 4 marker lists (up to 4096 markers one kernel
+ * does 0-4, and its time is in 0),
  * 5 interpolation and system assembly (one kernel; 6 is kept for the
  * assembly and reads 0), 7 implicit solve and spreading (one kernel; 8 is
  * kept for the spreading and reads 0),

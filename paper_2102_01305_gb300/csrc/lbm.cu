@@ -1070,7 +1070,7 @@ FluidParams<R> make_params(ibl_ctx* c, bool with_ib) {
 // 128-thread blocks).
 static dim3 cell_block(ibl_ctx* c, int n) {
   if (!c->collide_auto) return dim3(c->collide_bx, c->collide_by, 1);
-  if (c->N < 512LL * num_sms()) return dim3(32, 1, 1);
+  if (c->N < 512LL * num_sms() && c->ny <= 65535) return dim3(32, 1, 1);   // ny is the grid's y extent
   return (n + 63) / 64 * 64 > (n + 31) / 32 * 32 ? dim3(32, 4, 1) : dim3(64, 2, 1);
 }
 static dim3 cell_grid(ibl_ctx* c, dim3 b) {

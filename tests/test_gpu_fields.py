@@ -81,8 +81,9 @@ def test_collision_with_and_without_force(ibl, prec, force):
     assert rel_err(ctx.ibl_get_field(ibl.IBL_FIELD_U), sim.fields()[1]) < tol
 
 
-# 19 FP64 populations: just under 64 MB (one copy), just over, a ragged last chunk
-@pytest.mark.parametrize("shape", [(76, 76, 76), (76, 76, 77), (79, 81, 83)])
+# 19 FP64 populations: just under 16 MB (one copy), just over (two threads), a
+# ragged last chunk, all eight threads
+@pytest.mark.parametrize("shape", [(48, 48, 47), (48, 48, 49), (61, 53, 67), (79, 81, 83)])
 def test_large_host_transfers_round_trip(ibl, shape):
     """Exact round trip, four contexts' transfers at once from as many threads."""
     from concurrent.futures import ThreadPoolExecutor
