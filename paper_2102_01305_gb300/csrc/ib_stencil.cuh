@@ -156,7 +156,9 @@ __device__ __forceinline__ bool axis_stencil(double x, int n, bool per, int& bas
   }
   if (EXACT64) {
     double wd[4];
-    cosine_weights(x - floor(x), wd);
+    // fl, not floor(x): for x in (-2^-64, 0) the split rounds to node 0, where
+    // x - floor(x) rounds to 1, a node further on
+    cosine_weights(x - (double)fl, wd);
     for (int k = 0; k < 4; ++k) w[k] = df_from_double(wd[k]);
   } else {
     weights_df(t, w);
