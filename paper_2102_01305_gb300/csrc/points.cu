@@ -761,7 +761,7 @@ cudaError_t spread_points(ibl_ctx* c, int m, const double* X, const double* V, c
   if (m == 0) return cudaMemsetAsync(out, 0, sizeof(double) * (size_t)D * (size_t)c->N, c->stream);
   const PtGeo g = pt_geo(c);
   PtPlan plan;
-  cudaError_t e = point_plan<D>(c, m, X, V, ds, true, false, plan);
+  cudaError_t e = point_plan<D>(c, m, X, V, ds, true, c->prec == IBL_FP64, plan);
   if (e != cudaSuccess) return e;
   int* any_heavy = static_cast<int*>(c->d_pt_off) + g.tiles;
   unsigned char* heavy = reinterpret_cast<unsigned char*>(static_cast<int*>(c->d_pt_off) + 2 * (size_t)g.tiles + 2);

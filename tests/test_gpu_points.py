@@ -262,3 +262,33 @@ def test_interpolate_binned_order(ibl, q, prec, shape, bc):
     parts = [ctx.ibl_interpolate_points(_dev(X[k:k + part])) for k in range(0, m, part)]
     assert torch.equal(U, torch.cat([p[0] for p in parts]))
     assert torch.equal(rho, torch.cat([p[1] for p in parts]))
+
+
+def _weight_error(ibl, prec):
+    """Largest error of the spreading's x weights: points on nodes of y and z (weights 1/4 and 1/2, exact in
+    their products) and anywhere in x, far enough apart to share no cell; V ds is a power of two."""
+    nx, ny, nz = 96, 40, 40
+    ctx = ibl.from_workload({"lattice": 19, "tau": 0.7, "grid": W.grid(nx, ny, nz, [W.PERIODIC] * 6, precision=prec),
+                             "bodies": []}, init=False)
+    ix, iy, iz = (a.ravel() for a in np.meshgrid(np.arange(2, nx - 4, 6), np.arange(2, ny, 4), np.arange(2, nz, 4)))
+    s = np.random.default_rng(17).uniform(size=ix.size)
+    s[:8] = [0.0, 0.5, 2.0 ** -30, 1 - 2.0 ** -30, 0.25, 0.75, 2.0 ** -12, 1 - 2.0 ** -45]
+    X = np.stack([ix + s, iy, iz], axis=1).astype(np.float64)
+    V = np.zeros((ix.size, 3))
+    V[:, 0] = 2.0 ** 16
+    out = ctx.ibl_spread_points(_dev(X), _dev(V), _dev(np.ones(ix.size)))[0].cpu().numpy()
+    x = X[:, 0].astype(np.longdouble)
+    k = np.arange(-1, 3)
+    r = (x - ix)[:, None] - k
+    w = (1 + np.cos(np.longdouble("3.14159265358979323846264338327950288") / 2 * r)) / 4
+    got = out[iz[:, None], iy[:, None], ix[:, None] + k].astype(np.longdouble) / (2.0 ** 16 * 0.25)
+    return float(np.abs(got - w).max())
+
+
+# an FP64 evaluation (sincospi within 1 ulp, one addition): 0.25 (2^-53 + 2^-54); its double-float: half an
+# ulp of the low part under 2^-26, 2^-51; the fixed-point sums: 2 quanta in units of V ds / 4
+WEIGHT_BOUND = 0.25 * 1.5 * 2.0 ** -53 + 2.0 ** -51 + 2 * FIX_QUANTUM / 2.0 ** 14
+
+
+def test_spread_weights_fp64(ibl):
+    assert _weight_error(ibl, "fp64") <= WEIGHT_BOUND
