@@ -5,6 +5,7 @@
 
 #include "df.cuh"
 #include "lbm_gather.cuh"
+#include "stencil_fixed.cuh"
 
 namespace ibl {
 
@@ -40,84 +41,31 @@ __device__ __forceinline__ bool stencil_axis(double x, int n, bool per, int& bas
   return finite && fl - 1.0 >= 0.0 && fl + 2.0 < (double)n;
 }
 
-// First stencil node of a point at x on one axis and the position between
-// nodes, x - floor(x) - 1/2, as a 64-bit signed fraction (units of 2^-64), in
-// integer arithmetic on the bits of x: FP64 instructions issue at about 1/64
-// of the FP32 rate here.  False for |x| >= 2^31 and non-finite x, which take
-// the FP64 route (stencil_axis).
+// Floor and position between nodes of x (split_bits); false for |x| >= 2^31 and
+// non-finite x, which take the FP64 route (stencil_axis).
 __device__ __forceinline__ bool split_coordinate(double x, long long& fl, long long& t) {
-  const unsigned long long bits = (unsigned long long)__double_as_longlong(x);
-  const int e = (int)((bits >> 52) & 0x7ff) - 1023;
-  if (e >= 31) return false;
-  const unsigned long long mant = (bits & 0xfffffffffffffull) | (e > -1023 ? 0x10000000000000ull : 0ull);
-  long long ip = e >= 0 ? (long long)(mant >> (52 - e)) : 0;
-  const int sh = e + 12;
-  // fraction in units of 2^-64 (the integer bits leave the word)
-  unsigned long long f = sh >= 0 ? mant << sh : (sh > -64 ? mant >> -sh : 0ull);
-  if (bits >> 63) {
-    ip = -ip - (f != 0 ? 1 : 0);
-    f = 0ull - f;
-  }
-  fl = ip;
-  t = (long long)(f ^ 0x8000000000000000ull);
-  return true;
+  return split_bits((unsigned long long)__double_as_longlong(x), fl, t);
 }
 
-// The four weights of Eq. 14 from t = s - 1/2 (s = x - floor(x)) in
-// double-float arithmetic.  The nodes sit at |r| = 1+s, s, 1-s, 2-s, and with
-// p = pi t / 2 (|p| <= pi/4) the weights are 1/4 -/+ k (cos p + sin p) and
-// 1/4 +/- k (cos p - sin p), k = sqrt(2)/8.  k cos p and k sin p are the Taylor
-// polynomials in t^2 through p^16 and p^15 (remainder below 1e-17), the terms
-// below 1e-8 summed in FP32, the others in double-float.  Against 80-bit
-// arithmetic on 4e5 positions the weights are within 2.3e-15 (root mean square 4e-16; the
-// FP64 formula rounded to double-float: 4.9e-16 and 2e-16): under the products'
-// own rounding, and far under the spreading's resolution (1.4e-14) and FP32
-// storage.  FP64 storage keeps the FP64 formula for its interpolation.
-__device__ __forceinline__ df horner_step(df y, df p, df c) {
-  // c + y p with |y p| <= 0.32 |c|
-  const float q = __fmul_rn(y.hi, p.hi);
-  float e = fmaf(y.hi, p.hi, -q);
-  e = fmaf(y.hi, p.lo, e);
-  e = fmaf(y.lo, p.hi, e);
-  const float s = __fadd_rn(c.hi, q);
-  const float r = __fsub_rn(q, __fsub_rn(s, c.hi));
-  return fast_two_sum(s, __fadd_rn(r, __fadd_rn(e, c.lo)));
+// A weight in units of 2^-60 (at most 1/2) as a double-float: pieces of 24, 24
+// and 12 bits, the low part rounded once.
+__device__ __forceinline__ df df_from_fixed(long long w) {
+  const float h = __fmul_rn((float)(int)(w >> 36), 0x1p-24f);
+  const float m = __fmul_rn((float)(int)((w >> 12) & 0xffffff), 0x1p-48f);
+  const float l = __fmul_rn((float)(int)(w & 0xfff), 0x1p-60f);
+  const df s = fast_two_sum(h, m);
+  return fast_two_sum(s.hi, __fadd_rn(s.lo, l));
 }
 
-__device__ __forceinline__ df quarter_plus(df a) {
-  // 1/4 + a with |a| <= 1/4
-  const float s = __fadd_rn(0.25f, a.hi);
-  const float e = __fsub_rn(a.hi, __fsub_rn(s, 0.25f));
-  return fast_two_sum(s, __fadd_rn(e, a.lo));
-}
-
-__device__ __forceinline__ void weights_df(long long t64, df w[4]) {
-  const float h = (float)(int)(t64 >> 40), l = (float)(int)((t64 >> 16) & 0xffffff), r = (float)(int)(t64 & 0xffff);
-  const df t = fast_two_sum(__fmul_rn(h, 0x1p-24f), fmaf(r, 0x1p-64f, __fmul_rn(l, 0x1p-48f)));
-  const df y = df_mul(t, t);
-  // k sin(pi t / 2) = t P(y)
-  float u = fmaf(-0x1.03fcf0p-33f, y.hi, 0x1.59be1ep-27f);
-  u = fmaf(u, y.hi, -0x1.558d82p-21f);
-  df p = horner_step(y, df_make(u, 0.f), df_make(0x1.dbd6fep-16f, -0x1.52a032p-41f));
-  p = horner_step(y, p, df_make(-0x1.b1e9f4p-11f, 0x1.66adc2p-36f));
-  p = horner_step(y, p, df_make(0x1.cda106p-7f, 0x1.c1070cp-34f));
-  p = horner_step(y, p, df_make(-0x1.d3ba5cp-4f, -0x1.c5f47ep-32f));
-  p = horner_step(y, p, df_make(0x1.1c5832p-2f, -0x1.48a746p-28f));
-  const df s = df_mul(t, p);
-  // k cos(pi t / 2) = Q(y)
-  u = fmaf(0x1.986366p-37f, y.hi, -0x1.36567ep-30f);
-  u = fmaf(u, y.hi, 0x1.65ac58p-24f);
-  u = fmaf(u, y.hi, -0x1.2afa9ep-18f);
-  df c = horner_step(y, df_make(u, 0.f), df_make(0x1.54cb90p-13f, -0x1.5f0bbap-38f));
-  c = horner_step(y, c, df_make(-0x1.e36ab0p-9f, -0x1.827174p-34f));
-  c = horner_step(y, c, df_make(0x1.6f5a4ap-5f, -0x1.35a078p-31f));
-  c = horner_step(y, c, df_make(-0x1.bea5b6p-3f, -0x1.cac988p-33f));
-  c = horner_step(y, c, df_make(0x1.6a09e6p-3f, 0x1.9fcef4p-29f));
-  const df a = df_add(c, s), b = df_sub(c, s);   // k (cos + sin), k (cos - sin)
-  w[0] = quarter_plus(df_neg(a));
-  w[1] = quarter_plus(b);
-  w[2] = quarter_plus(a);
-  w[3] = quarter_plus(df_neg(b));
+// The four weights as double-floats (fixed_weights).  Against 64-bit-mantissa
+// arithmetic at 2e4 positions they err by at most 4.4e-16 (root mean square
+// 1.43e-16), the FP64 formula rounded to double-float by 5.1e-16 (1.46e-16), and
+// a polynomial in double-float by 2.3e-15 (4e-16).
+__device__ __forceinline__ void weights_df(long long t, df w[4]) {
+  long long f[4];
+  fixed_weights(t, f);
+#pragma unroll
+  for (int k = 0; k < 4; ++k) w[k] = df_from_fixed(f[k]);
 }
 
 // First stencil node of one axis, wrapped into [0, n) on a periodic axis;

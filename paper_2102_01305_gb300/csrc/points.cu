@@ -128,7 +128,8 @@ __global__ void __launch_bounds__(1024) k_pt_scan(int n, const int* __restrict__
 // Records and weights in bin order (slot == nullptr: in the given order), and
 // for the spreading V_l ds_l 2^46 as double-floats.  rec = (first nodes, point);
 // a point whose stencil fails gets first node -1 and is left out later.
-// EXACT64: the weights from the FP64 formula.
+// EXACT64: the weights from the FP64 formula (interpolation in FP64 contexts),
+// else in integers, which err by less.
 template <int D, bool EXACT64>
 __global__ void k_pt_records(int m, const double* __restrict__ X, PtGeo g, const int2* __restrict__ slot,
                              const int* __restrict__ off, int4* __restrict__ rec, df* __restrict__ wts,
@@ -761,7 +762,7 @@ cudaError_t spread_points(ibl_ctx* c, int m, const double* X, const double* V, c
   if (m == 0) return cudaMemsetAsync(out, 0, sizeof(double) * (size_t)D * (size_t)c->N, c->stream);
   const PtGeo g = pt_geo(c);
   PtPlan plan;
-  cudaError_t e = point_plan<D>(c, m, X, V, ds, true, c->prec == IBL_FP64, plan);
+  cudaError_t e = point_plan<D>(c, m, X, V, ds, true, false, plan);
   if (e != cudaSuccess) return e;
   int* any_heavy = static_cast<int*>(c->d_pt_off) + g.tiles;
   unsigned char* heavy = reinterpret_cast<unsigned char*>(static_cast<int*>(c->d_pt_off) + 2 * (size_t)g.tiles + 2);

@@ -292,3 +292,9 @@ WEIGHT_BOUND = 0.25 * 1.5 * 2.0 ** -53 + 2.0 ** -51 + 2 * FIX_QUANTUM / 2.0 ** 1
 
 def test_spread_weights_fp64(ibl):
     assert _weight_error(ibl, "fp64") <= WEIGHT_BOUND
+
+
+@pytest.mark.parametrize("prec", ["fp32", "fp16dev", "bf16dev"])
+def test_spread_weights_of_integer_polynomials(ibl, prec):
+    """FP32 and 16-bit contexts form the weights in integer arithmetic (2^-60): held to the FP64 formula's bound."""
+    assert _weight_error(ibl, prec) <= WEIGHT_BOUND
