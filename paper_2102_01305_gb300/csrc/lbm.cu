@@ -883,15 +883,16 @@ __global__ void __launch_bounds__(256) k_fields(const T* __restrict__ src, Fluid
         if (c[a] != 0) m[a] = c[a] > 0 ? O::add(m[a], gi) : O::sub(m[a], gi);
     }
   }
-  if (sizeof(R) == 4 && !isfinite(O::value(drho))) {
-    // double-float turns an infinity into a NaN: such a cell in plain FP64
+  if (!isfinite(O::value(drho))) {
+    // double-float turns an infinity into a NaN: such a cell in plain FP64, term
+    // by term, where an infinity makes every component of u a NaN
     double r = 0.0, q[3] = {0.0, 0.0, 0.0};
     for (int i = 0; i < Q; ++i) {
       const double gi = (double)g[i];
       r += gi;
-      if (Lat<Q>::cx(i)) q[0] += Lat<Q>::cx(i) * gi;
-      if (Lat<Q>::cy(i)) q[1] += Lat<Q>::cy(i) * gi;
-      if (Lat<Q>::cz(i)) q[2] += Lat<Q>::cz(i) * gi;
+      q[0] += Lat<Q>::cx(i) * gi;
+      q[1] += Lat<Q>::cy(i) * gi;
+      q[2] += Lat<Q>::cz(i) * gi;
     }
     if (rho_out) rho_out[cell] = 1.0 + r;
     if (U)

@@ -110,3 +110,15 @@ def test_force_history_ring(ibl):
     whole = ctx.ibl_force_history(0, 9)
     assert len(whole) == 9 and np.array_equal(ctx.ibl_force_history(0, 100), whole)
     assert np.array_equal(ctx.ibl_force_history(0, 4), whole[5:]) and len(ctx.ibl_force_history(0, 0)) == 0
+
+
+@pytest.mark.parametrize("prec", ["fp64", "fp32"])
+def test_velocity_of_infinite_populations(ibl, prec):
+    """u = sum c_i f_i / rho with an infinite f_0 is no number in any component (0 * inf)."""
+    q, shape = 19, (8, 8, 8)
+    f = np.tile(get_lattice(q).w[:, None, None, None], (1,) + shape)
+    f[0, 3, 4, 5] = np.inf
+    ctx = _ctx(ibl, q, shape, prec)
+    ctx.ibl_set_populations(f)
+    u = ctx.ibl_get_field(ibl.IBL_FIELD_U)
+    assert np.isnan(u[:, 3, 4, 5]).all() and np.count_nonzero(np.isnan(u)) == 3
