@@ -814,50 +814,39 @@ __global__ void __launch_bounds__(TILE_CELLS) k_collide_band(DirPtrs<Q, T> P, Fl
   }
 }
 
-// Sums over one cell's populations beyond the storage's precision.  FP64
-// storage sums in FP64.  FP32 and 16-bit storage sum in double-float (48 bits,
-// the storage has 24 at most): FP64 instructions, conversions included, issue at
-// about 1/64 of the FP32 rate, and the kernels that used them here were bound by
-// them.
-template <class R> struct Wide;
-template <> struct Wide<double> {
-  using V = double;
-  static __device__ __forceinline__ V of(double a) { return a; }
-  static __device__ __forceinline__ V add(V a, V b) { return a + b; }
-  static __device__ __forceinline__ V sub(V a, V b) { return a - b; }
-  static __device__ __forceinline__ V mul(V a, V b) { return a * b; }
-  static __device__ __forceinline__ V div(V a, V b) { return a / b; }
-  static __device__ __forceinline__ double value(V a) { return a; }
-  static __device__ __forceinline__ double store(V a) { return a; }
-  static __device__ __forceinline__ V konst(double c) { return c; }
+// Sum of one cell's populations to FP64's accuracy.  FP64 storage sums in FP64.
+// FP32 and 16-bit storage keep the sum and its rounding errors in three FP32
+// numbers (TwoSum: exact up to 2^-72 of the terms), so that FP64 arithmetic,
+// which issues at about 1/64 of the FP32 rate and bounded these kernels, is left
+// with three conversions a sum.
+template <class R> struct CellSum;
+template <> struct CellSum<double> {
+  double v = 0.0;
+  __device__ __forceinline__ void add(double a) { v += a; }
+  __device__ __forceinline__ bool finite() const { return isfinite(v); }
+  __device__ __forceinline__ double value() const { return v; }
 };
-template <> struct Wide<float> {
-  using V = df;
-  static __device__ __forceinline__ V of(float a) { return df_make(a, 0.f); }
-  static __device__ __forceinline__ V of(double a) { return df_from_double(a); }
-  // one rounding of the low parts: an error of about 2^-47 of the larger operand
-  static __device__ __forceinline__ V add(V a, V b) {
-    const df s = two_sum(a.hi, b.hi);
-    return fast_two_sum(s.hi, __fadd_rn(s.lo, __fadd_rn(a.lo, b.lo)));
+template <> struct CellSum<float> {
+  float s = 0.f, c = 0.f, d = 0.f;
+  __device__ __forceinline__ void add(float a) {
+    const df t = two_sum(s, a), e = two_sum(c, t.lo);
+    s = t.hi;
+    c = e.hi;
+    d = __fadd_rn(d, e.lo);
   }
-  static __device__ __forceinline__ V sub(V a, V b) { return add(a, df_neg(b)); }
-  static __device__ __forceinline__ V mul(V a, V b) { return df_mul(a, b); }
-  static __device__ __forceinline__ V div(V a, V b) { return df_div(a, b); }
-  static __device__ __forceinline__ double value(V a) { return df_to_double(a); }
-  static __device__ __forceinline__ float store(V a) { return a.hi; }   // normalised: hi is the rounded value
-  static __device__ __forceinline__ V konst(double c) { return df_make((float)c, (float)(c - (double)(float)c)); }
+  // an infinity or an overflow leaves a NaN in c
+  __device__ __forceinline__ bool finite() const { return isfinite(c); }
+  __device__ __forceinline__ double value() const { return ((double)c + (double)d) + (double)s; }
 };
 
 // rho, u = (sum c_i f_i + G/2)/rho and optionally f itself (FP64) of the
 // current post-streaming populations.  U: the velocity is asked for.
-// 64^3 FP32: 68 us for u with FP64 sums and divisions, 14 us now.
+// 64^3 FP32: 68 us for u when every population is converted to FP64.
 template <int Q, class T, bool PULL, bool U>
 __global__ void __launch_bounds__(256) k_fields(const T* __restrict__ src, FluidParams<typename Store<T>::R> p,
                                                 double* __restrict__ rho_out, double* __restrict__ u_out,
                                                 double* __restrict__ pop_out) {
   using R = typename Store<T>::R;
-  using O = Wide<R>;
-  using V = typename O::V;
   const int x = blockIdx.x * blockDim.x + threadIdx.x;
   const int y = blockIdx.y * blockDim.y + threadIdx.y;
   const int z = blockIdx.z;
@@ -870,45 +859,69 @@ __global__ void __launch_bounds__(256) k_fields(const T* __restrict__ src, Fluid
     for (int i = 0; i < Q; ++i) pop_out[i * p.N + cell] = (double)g[i] + Lat<Q>::w(i);
   }
   if (!rho_out && !U) return;
-  V drho = O::of(g[0]);
-  V m[3] = {O::of(p.G[0] * R(0.5)), O::of(p.G[1] * R(0.5)), O::of(p.G[2] * R(0.5))};
+  CellSum<R> sum, ms[3];
 #pragma unroll
-  for (int i = 1; i < Q; ++i) {
-    const V gi = O::of(g[i]);
-    drho = O::add(drho, gi);
+  for (int i = 0; i < Q; ++i) {
+    sum.add(g[i]);
     if (U) {
       const int c[3] = {Lat<Q>::cx(i), Lat<Q>::cy(i), Lat<Q>::cz(i)};
 #pragma unroll
       for (int a = 0; a < 3; ++a)
-        if (c[a] != 0) m[a] = c[a] > 0 ? O::add(m[a], gi) : O::sub(m[a], gi);
+        if (c[a] != 0) ms[a].add(c[a] > 0 ? g[i] : -g[i]);
     }
   }
-  if (!isfinite(O::value(drho))) {
-    // double-float turns an infinity into a NaN: such a cell in plain FP64, term
-    // by term, where an infinity makes every component of u a NaN
-    double r = 0.0, q[3] = {0.0, 0.0, 0.0};
+  double drho = 0.0, m[3] = {0.0, 0.0, 0.0};
+  if (sum.finite() && (!U || (ms[0].finite() && ms[1].finite() && ms[2].finite()))) {
+    drho = sum.value();
+    if (U) {
+#pragma unroll
+      for (int a = 0; a < Lat<Q>::D; ++a) m[a] = ms[a].value();
+    }
+  } else {   // term by term in FP64 (an infinity makes every component of u a NaN)
     for (int i = 0; i < Q; ++i) {
       const double gi = (double)g[i];
-      r += gi;
-      q[0] += Lat<Q>::cx(i) * gi;
-      q[1] += Lat<Q>::cy(i) * gi;
-      q[2] += Lat<Q>::cz(i) * gi;
+      drho += gi;
+      m[0] += Lat<Q>::cx(i) * gi;
+      m[1] += Lat<Q>::cy(i) * gi;
+      m[2] += Lat<Q>::cz(i) * gi;
     }
-    if (rho_out) rho_out[cell] = 1.0 + r;
-    if (U)
-      for (int a = 0; a < Lat<Q>::D; ++a) u_out[a * p.N + cell] = (q[a] + 0.5 * (double)p.G[a]) / (1.0 + r);
-    return;
   }
-  const V rho = O::add(O::konst(1.0), drho);
-  if (rho_out) rho_out[cell] = 1.0 + O::value(drho);
+  const double rho = 1.0 + drho;
+  if (rho_out) rho_out[cell] = rho;
   if (U) {
-    // double-float: one division and a product per component
-    const V inv = sizeof(R) == 4 ? O::div(O::konst(1.0), rho) : rho;
 #pragma unroll
-    for (int a = 0; a < Lat<Q>::D; ++a)
-      u_out[a * p.N + cell] = O::value(sizeof(R) == 4 ? O::mul(m[a], inv) : O::div(m[a], rho));
+    for (int a = 0; a < Lat<Q>::D; ++a) {
+      if (p.G[a] != R(0)) m[a] += 0.5 * (double)p.G[a];
+      u_out[a * p.N + cell] = m[a] / rho;
+    }
   }
 }
+
+// Arithmetic of the initial state: FP64, or double-float for FP32 and 16-bit
+// storage.
+template <class R> struct Wide;
+template <> struct Wide<double> {
+  using V = double;
+  static __device__ __forceinline__ V of(double a) { return a; }
+  static __device__ __forceinline__ V add(V a, V b) { return a + b; }
+  static __device__ __forceinline__ V sub(V a, V b) { return a - b; }
+  static __device__ __forceinline__ V mul(V a, V b) { return a * b; }
+  static __device__ __forceinline__ double store(V a) { return a; }
+  static __device__ __forceinline__ V konst(double c) { return c; }
+};
+template <> struct Wide<float> {
+  using V = df;
+  static __device__ __forceinline__ V of(double a) { return df_from_double(a); }
+  // one rounding of the low parts: an error of about 2^-47 of the larger operand
+  static __device__ __forceinline__ V add(V a, V b) {
+    const df s = two_sum(a.hi, b.hi);
+    return fast_two_sum(s.hi, __fadd_rn(s.lo, __fadd_rn(a.lo, b.lo)));
+  }
+  static __device__ __forceinline__ V sub(V a, V b) { return add(a, df_neg(b)); }
+  static __device__ __forceinline__ V mul(V a, V b) { return df_mul(a, b); }
+  static __device__ __forceinline__ float store(V a) { return a.hi; }   // normalised: hi is the rounded value
+  static __device__ __forceinline__ V konst(double c) { return df_make((float)c, (float)(c - (double)(float)c)); }
+};
 
 // f_i = f_eq(rho, u) - w_i (Eq. 4), by direction pairs (c, -c) that share the
 // even part: w [drho + rho (4.5 cu^2 - 1.5 u.u)] +/- w rho 3 cu.
@@ -978,15 +991,14 @@ __global__ void k_set_pop(T* __restrict__ dst, long long N, const double* __rest
 
 // Fixed-order mass: block b sums cells [b*chunk, (b+1)*chunk) in a fixed
 // strided pattern and a fixed tree; the host-side second pass is a fixed loop.
-// A cell's deviations are summed beyond the storage's precision (Wide), the
-// cells' sums in FP64, and the cells themselves are counted.  Bound by HBM in
+// A cell's deviations are summed to FP64's accuracy (CellSum), the cells' sums
+// in FP64, and the cells themselves are counted.  Bound by HBM in
 // FP32 (256^3: 268 us; 1280 us with FP64 conversions and additions per
 // direction and 64-bit index divisions).
 template <int Q, class T, bool PULL>
 __global__ void __launch_bounds__(256) k_mass(const T* __restrict__ src, FluidParams<typename Store<T>::R> p,
                                               double* __restrict__ partials, long long chunk) {
   using R = typename Store<T>::R;
-  using O = Wide<R>;
   __shared__ double sh[256];
   const long long start = (long long)blockIdx.x * chunk;
   long long end = start + chunk;
@@ -999,12 +1011,13 @@ __global__ void __launch_bounds__(256) k_mass(const T* __restrict__ src, FluidPa
     const unsigned z = yz / (unsigned)p.ny;
     R g[Q];
     pull_cell<Q, T, PULL>(src, (int)(cell - yz * (unsigned)p.nx), (int)(yz - z * (unsigned)p.ny), (int)z, p, g);
-    typename O::V drho = O::of(g[0]);
+    CellSum<R> sum;
 #pragma unroll
-    for (int i = 1; i < Q; ++i) drho = O::add(drho, O::of(g[i]));
-    double cell_sum = O::value(drho);
-    if (sizeof(R) == 4 && !isfinite(cell_sum)) {   // an infinity, which double-float turns into a NaN
-      cell_sum = 0.0;
+    for (int i = 0; i < Q; ++i) sum.add(g[i]);
+    double cell_sum = 0.0;
+    if (sum.finite()) {
+      cell_sum = sum.value();
+    } else {   // an infinity, or an overflow in FP32
       for (int i = 0; i < Q; ++i) cell_sum += (double)g[i];
     }
     acc += cell_sum;

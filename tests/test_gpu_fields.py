@@ -122,3 +122,23 @@ def test_velocity_of_infinite_populations(ibl, prec):
     ctx.ibl_set_populations(f)
     u = ctx.ibl_get_field(ibl.IBL_FIELD_U)
     assert np.isnan(u[:, 3, 4, 5]).all() and np.count_nonzero(np.isnan(u)) == 3
+
+
+@pytest.mark.parametrize("prec", list(UNIT))
+@pytest.mark.parametrize("q,shape", SHAPES)
+def test_readout_to_fp64_accuracy(ibl, q, shape, prec):
+    """rho and u of given populations as FP64 forms them: 1 + drho and the division round once each (2^-53
+    relative), the sums are exact.  The deviations are multiples of 2^-13 (FP32: 2^-30) that every storage holds."""
+    lat = get_lattice(q)
+    rng = np.random.default_rng(12)
+    top, unit = (2 ** 22, 2.0 ** -30) if prec == "fp32" else (127, 2.0 ** -14)
+    k = rng.integers(-top, top + 1, size=(q,) + shape)
+    ctx = _ctx(ibl, q, shape, prec)
+    f = np.empty((q,) + shape)
+    f[gpu_to_oracle_order(ibl, q)] = lat.w[:, None, None, None] + unit * k
+    ctx.ibl_set_populations(f)
+    rho, u = ctx.ibl_get_field(ibl.IBL_FIELD_RHO), ctx.ibl_get_field(ibl.IBL_FIELD_U)
+    want_rho = np.longdouble(1) + k.sum(axis=0).astype(np.longdouble) * np.longdouble(unit)
+    m = np.tensordot(np.asarray(lat.c)[:, :lat.d].T, k, axes=1).astype(np.longdouble) * np.longdouble(unit)
+    assert (np.abs(rho - want_rho) <= 2.0 ** -53 * want_rho * 1.01).all()
+    assert (np.abs(u - m / want_rho) <= 2.02 * 2.0 ** -53 * np.abs(m / want_rho)).all()
