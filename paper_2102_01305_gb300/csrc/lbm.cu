@@ -908,6 +908,8 @@ template <> struct Wide<double> {
   static __device__ __forceinline__ V mul(V a, V b) { return a * b; }
   static __device__ __forceinline__ double store(V a) { return a; }
   static __device__ __forceinline__ V konst(double c) { return c; }
+  static __device__ __forceinline__ double error(V, V, const V*) { return 0.0; }
+  static __device__ __forceinline__ bool rounds(V, double) { return true; }
 };
 template <> struct Wide<float> {
   using V = df;
@@ -921,11 +923,35 @@ template <> struct Wide<float> {
   static __device__ __forceinline__ V mul(V a, V b) { return df_mul(a, b); }
   static __device__ __forceinline__ float store(V a) { return a.hi; }   // normalised: hi is the rounded value
   static __device__ __forceinline__ V konst(double c) { return df_make((float)c, (float)(c - (double)(float)c)); }
+  // bound of f_eq's double-float error over w (rho3 = 3 rho), twice over
+  static __device__ __forceinline__ float error(V drho, V rho3, const V u[3]) {
+    const float s = fabsf(u[0].hi) + fabsf(u[1].hi) + fabsf(u[2].hi);
+    return 0x1p-41f * (fabsf(drho.hi) + fabsf(rho3.hi) * s * (1.f + 2.f * s));
+  }
+  // whether every value within e of a (and within the products' underflow) has a's rounding to FP32
+  static __device__ __forceinline__ bool rounds(V a, float e) {
+    if (a.hi == 0.f && e == 0.f) return true;
+    e += 0x1p-140f;
+    return __fadd_rn(a.hi, __fadd_rn(a.lo, e)) == a.hi && __fadd_rn(a.hi, __fsub_rn(a.lo, e)) == a.hi;
+  }
 };
+
+// f_eq - w of direction i (Eq. 4) in FP64.
+template <int Q>
+__device__ __noinline__ double init_fp64(int i, double rho, double u0, double u1, double u2) {
+  const double cu = Lat<Q>::cx(i) * u0 + Lat<Q>::cy(i) * u1 + Lat<Q>::cz(i) * u2;
+  const double usq = u0 * u0 + u1 * u1 + u2 * u2;
+  return Lat<Q>::w(i) * ((rho - 1.0) + rho * (3.0 * cu + 4.5 * cu * cu - 1.5 * usq));
+}
 
 // f_i = f_eq(rho, u) - w_i (Eq. 4), by direction pairs (c, -c) that share the
 // even part: w [drho + rho (4.5 cu^2 - 1.5 u.u)] +/- w rho 3 cu.
 // GIVEN = false: at rest with rho = 1 the deviations are zero.
+// FP32 and 16-bit storage form it in double-float, whose error is below w 2^-42
+// (|drho| + rho (3 U + 6 U^2)), U = sum |u_a| (each of the ten operations errs by
+// at most 2^-45 of its terms); a value whose rounding to FP32 that error could
+// change (about 1 in 1e4), or that is not finite, is formed in FP64 instead, so
+// the stored values are those of FP64 arithmetic.
 // Bound by FP64 conversions of the given field and, in FP32, by HBM: 256^3
 // FP32 413 us, 5189 us when every direction was formed in FP64 by itself.
 template <int Q, class T, bool GIVEN>
@@ -941,25 +967,29 @@ __global__ void __launch_bounds__(256) k_init_eq(T* __restrict__ dst, long long 
     for (int i = 0; i < Q; ++i) dst[i * N + cell] = Store<T>::st(R(0));
     return;
   }
-  V u[3] = {O::konst(0.0), O::konst(0.0), O::konst(0.0)};
-  if (u_in) {
-#pragma unroll
-    for (int a = 0; a < Lat<Q>::D; ++a) u[a] = O::of(u_in[a * N + cell]);
-  }
+  const double ud[3] = {u_in ? u_in[cell] : 0.0, u_in ? u_in[N + cell] : 0.0,
+                        u_in && Lat<Q>::D == 3 ? u_in[2 * N + cell] : 0.0};
+  const double rd = rho_in ? rho_in[cell] : 1.0;
+  const V u[3] = {O::of(ud[0]), O::of(ud[1]), O::of(ud[2])};
   V usq = O::add(O::mul(u[0], u[0]), O::mul(u[1], u[1]));
   if (Lat<Q>::D == 3) usq = O::add(usq, O::mul(u[2], u[2]));
   V drho = O::konst(0.0);
   V rho3 = O::konst(3.0), rho45 = O::konst(4.5), rho15 = O::konst(-1.5);
   if (rho_in) {
-    const double r = rho_in[cell];
-    const V rv = O::of(r);
-    drho = O::of(r - 1.0);
+    const V rv = O::of(rd);
+    drho = O::of(rd - 1.0);
     rho3 = O::mul(rho3, rv);
     rho45 = O::mul(rho45, rv);
     rho15 = O::mul(rho15, rv);
   }
   const V base = O::add(drho, O::mul(rho15, usq));
-  dst[cell] = Store<T>::st((R)O::store(O::mul(O::konst(Lat<Q>::w(0)), base)));
+  const R err = O::error(drho, rho3, u);
+  const auto put = [&](int i, V v) {
+    R r = (R)O::store(v);
+    if (!O::rounds(v, R(Lat<Q>::w(i)) * err)) r = (R)init_fp64<Q>(i, rd, ud[0], ud[1], ud[2]);
+    dst[i * N + cell] = Store<T>::st(r);
+  };
+  put(0, O::mul(O::konst(Lat<Q>::w(0)), base));
 #pragma unroll
   for (int i = 1; i < Q; i += 2) {
     // c.u of the first member of a pair: its first nonzero component is +1
@@ -975,8 +1005,8 @@ __global__ void __launch_bounds__(256) k_init_eq(T* __restrict__ dst, long long 
     const V w = O::konst(Lat<Q>::w(i));
     const V even = O::add(base, O::mul(rho45, O::mul(cu, cu)));
     const V odd = O::mul(rho3, cu);
-    dst[i * N + cell] = Store<T>::st((R)O::store(O::mul(w, O::add(even, odd))));
-    dst[(i + 1) * N + cell] = Store<T>::st((R)O::store(O::mul(w, O::sub(even, odd))));
+    put(i, O::mul(w, O::add(even, odd)));
+    put(i + 1, O::mul(w, O::sub(even, odd)));
   }
 }
 

@@ -142,3 +142,22 @@ def test_readout_to_fp64_accuracy(ibl, q, shape, prec):
     m = np.tensordot(np.asarray(lat.c)[:, :lat.d].T, k, axes=1).astype(np.longdouble) * np.longdouble(unit)
     assert (np.abs(rho - want_rho) <= 2.0 ** -53 * want_rho * 1.01).all()
     assert (np.abs(u - m / want_rho) <= 2.02 * 2.0 ** -53 * np.abs(m / want_rho)).all()
+
+
+@pytest.mark.parametrize("q,shape", [(19, (160, 160, 160)), (9, (1, 1500, 2001))])
+def test_init_rounds_as_fp64(ibl, q, shape):
+    """FP32 storage holds f_eq - w as FP64 forms it, rounded once.  With velocities of 20 bits every FP64 operation
+    but the last product is exact, so the FP32 values are determined."""
+    d = get_lattice(q).d
+    u = np.random.default_rng(21).integers(-2 ** 19, 2 ** 19 + 1, size=(d,) + shape) * 2.0 ** -23
+    ctx = _ctx(ibl, q, shape, "fp32")
+    ctx.ibl_init_fluid(None, u)
+    f = ctx.ibl_get_populations()
+    c, w = ibl.lattice_velocities(q)
+    usq = (u * u).sum(axis=0)
+    for i in range(q):
+        cu = sum(int(c[i][a]) * u[a] for a in range(d))
+        g = w[i] * (3 * cu + 4.5 * cu * cu - 1.5 * usq)
+        # f was read as g + w in FP64, which holds all of g above 2^-20
+        large = np.abs(g) > 2.0 ** -20
+        assert np.array_equal((f[i] - w[i]).astype(np.float32)[large], g.astype(np.float32)[large])
