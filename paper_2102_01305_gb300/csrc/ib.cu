@@ -538,7 +538,24 @@ struct AssembleArgs {
   const int* ncand;
   const int* use_tiles;
   const int* cand_bad;
+  int* count;            // the tiles' marker counts, zero unless k_ib_front has made lists
 };
+
+// A tile with more markers than its list may hold is refused whether the lists
+// are read or not.  k_ib_front checks the lists that it makes; without lists a
+// tile's markers are counted here, one thread per (marker, touched tile) in blocks
+// of their own, off the critical path (in k_ib_front the count took 10 us of a step
+// at 1552 markers, by the interpolation's warps 5 at 3152).  A tile is then one
+// body's, so only bodies of more than TILE_MARKER_CAP markers need it.
+__device__ __forceinline__ void count_tile_markers(int e, int m_total, const int* __restrict__ base, const Geo& g,
+                                                   const AssembleArgs& aa) {
+  const int l = e >> 3, i = e & 7;
+  if (l >= m_total || *aa.use_tiles || *aa.cand_bad) return;
+  int t[8];
+  if (i >= touched_tiles(g, base + 3 * l, t)) return;
+  const int s = aa.tile_slot[t[i]];
+  if (s >= 0 && atomicAdd(&aa.count[s], 1) >= TILE_MARKER_CAP) atomicOr(aa.status, ST_OVERFLOW);
+}
 
 template <int Q, class T, bool PULL>
 __global__ void __launch_bounds__(256) k_interp_assemble(int nb_interp, int m_total, const int* __restrict__ base,
@@ -548,6 +565,8 @@ __global__ void __launch_bounds__(256) k_interp_assemble(int nb_interp, int m_to
                                                          double* __restrict__ B, AssembleArgs aa) {
   if ((int)blockIdx.x < nb_interp) {
     interpolate_body<Q, T, PULL>(blockIdx.x, m_total, base, wts, src, p, g, U, rho_l, B);
+  } else if ((int)blockIdx.x >= nb_interp + (m_total + 7) / 8) {
+    count_tile_markers(((int)blockIdx.x - nb_interp - (m_total + 7) / 8) * 256 + threadIdx.x, m_total, base, g, aa);
   } else {
     assemble_body(blockIdx.x - nb_interp, m_total, base, wts, aa.tile_slot, aa.tile_mcount, aa.tile_markers, g,
                   aa.body_of, aa.Gcol, aa.Gval, aa.Gnnz, aa.rowsum_max, aa.status, aa.cand, aa.ncand,
@@ -2318,12 +2337,17 @@ static cudaError_t interpolate_q(ibl_ctx* c, const Geo& g) {
   aa.ncand = c->d_ncand;
   aa.use_tiles = c->d_mixed;
   aa.cand_bad = c->d_mixed + 1;
+  aa.count = c->d_tile_mcount;
+  int cb = 0;                            // counting blocks
+  if (m <= FRONT_MARKERS)
+    for (auto& b : c->bodies)
+      if (b.m > TILE_MARKER_CAP) cb = (8 * m + 255) / 256;
   const df* w = reinterpret_cast<const df*>(c->d_wts);
   if (c->poststream)
-    k_interp_assemble<Q, T, false><<<wb + ab, 256, 0, c->stream>>>(wb, m, c->d_base, w, src, p, g, c->d_U, c->d_rho_l,
+    k_interp_assemble<Q, T, false><<<wb + ab + cb, 256, 0, c->stream>>>(wb, m, c->d_base, w, src, p, g, c->d_U, c->d_rho_l,
                                                                      c->d_B, aa);
   else
-    k_interp_assemble<Q, T, true><<<wb + ab, 256, 0, c->stream>>>(wb, m, c->d_base, w, src, p, g, c->d_U, c->d_rho_l,
+    k_interp_assemble<Q, T, true><<<wb + ab + cb, 256, 0, c->stream>>>(wb, m, c->d_base, w, src, p, g, c->d_U, c->d_rho_l,
                                                                     c->d_B, aa);
   c->launches++;
   return cudaGetLastError();

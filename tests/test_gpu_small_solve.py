@@ -55,3 +55,25 @@ def test_one_marker_and_moving_band(ibl):
     compare_fields(ctx, sim, ibl, TOL_FIELD_FP64)
     force = ctx.ibl_get_field(ibl.IBL_FIELD_FORCE)
     assert 0 < np.count_nonzero(force[0]) <= 16   # only the last step's stencil
+
+
+def test_marker_list_capacity_without_lists(ibl):
+    """576 markers of one still body on one 16 x 16 tile (a list holds 512): refused at the first step, although
+    nothing reads the lists of a single body."""
+    g = 14.1 + 0.79 * np.arange(24)
+    X0 = np.stack([a.ravel() for a in np.meshgrid(g, g)], axis=1)
+    still = {"kind": W.WAVE_CONST, "amp": 0.0, "offset": 0.0}
+    body = {"X0": X0, "ds": np.ones(len(X0)), "hinge": (0, 0, 0), "axis": (0, 0, 1), "origin": (0.0, 0.0, 0.0),
+            "A": still, "alpha": still, "beta": 0.0, "phi": 0.0, "f": 1 / 300.0, "J": 0.0}
+    cfg = {"lattice": 9, "tau": 0.8, "grid": W.grid(48, 48, 1, [W.PERIODIC] * 6, precision="fp64"), "bodies": [body],
+           "u0": (0.0, 0.0, 0.0), "reference": {"U_ref": 0.1, "L": 1.0, "rho_ref": 1.0}}
+    ctx = ibl.from_workload(cfg)
+    with pytest.raises(ibl.IblError, match="IBL_EINVAL"):
+        ctx.ibl_step(1)
+        ctx.ibl_sync()
+    # 528 markers at 1.5 lattice units spread over nine tiles: the same calls run
+    body["X0"] = np.stack([a.ravel() for a in np.meshgrid(6.0 + 1.5 * np.arange(22), 6.0 + 1.5 * np.arange(24))], axis=1)
+    body["ds"] = np.ones(len(body["X0"]))
+    ok = ibl.from_workload(cfg)
+    ok.ibl_step(1)
+    ok.ibl_sync()
