@@ -27,6 +27,7 @@
 #include <cooperative_groups.h>
 
 #include <cmath>
+#include <mutex>
 
 #include "df.cuh"
 #include "ib_stencil.cuh"
@@ -40,8 +41,10 @@ constexpr int MAX_BODIES = 16;
 constexpr int GJ_NB = 64;          // Gauss-Jordan pivot block
 constexpr int PCG_MAX_ITERS = 200;
 // Marker sets whose kinematics and band run on one cluster (at 3152 markers 34 us
-// between events a step, 41 as separate kernels), and those whose solve does (an iteration takes 3.9 us at 68 markers, 7.6 at 520 and 18 at 1140,
-// where G and M no longer fit the shared memory; k_pcg 12.4, 13.2 and 13.7).
+// between events a step, 41 as separate kernels), and those whose solve does (an
+// iteration takes 3.9 us at 68 markers, 7.6 at 520 and 18 at 1140, where G and M
+// no longer fit the shared memory; k_pcg 12.4, 13.2 and 13.7.  Whole steps of 608
+// markers, on sixteen blocks, in 80^3 FP32 cells: 134 us, with k_pcg 172).
 constexpr int FRONT_MARKERS = 4096;
 constexpr int CLUSTER_MARKERS = 640;
 // relative preconditioned residual (the spread field's A-norm error) per
@@ -2451,6 +2454,20 @@ static void body_state(const Body& B, double t, double st[8]) {
   st[7] = al;
 }
 
+// Launch of one cluster of `blocks` blocks.
+static void cluster_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute* at, int blocks, int threads, size_t smem,
+                           cudaStream_t stream) {
+  cfg.gridDim = dim3(blocks);
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = blocks;
+  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+}
+
 // Kinematics and the band tiles of the step (the bulk collide may start
 // once these are enqueued).
 cudaError_t ib_step_front(ibl_ctx* c) {
@@ -2507,15 +2524,8 @@ cudaError_t ib_step_front(ibl_ctx* c) {
     // one block up to 128 markers; eight above, for their FP64 units
     const int blocks = m <= 128 ? 1 : 8, threads = m <= 512 ? 256 : 512;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(blocks);
-    cfg.blockDim = dim3(threads);
-    cfg.stream = c->stream;
     cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = blocks;
-    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
+    cluster_config(cfg, at, blocks, threads, 0, c->stream);
     IBL_CU(cudaLaunchKernelEx(&cfg, c->prec == IBL_FP64 ? k_ib_front<true> : k_ib_front<false>, bt, M, g, F));
     for (int ph = 0; ph < 4; ++ph) phase_mark(c, ph);
     c->launches++;
@@ -2543,6 +2553,36 @@ cudaError_t ib_step_front(ibl_ctx* c) {
 // 1 to 16.
 // G and M stay in shared memory when they fit, else they are read from L2.
 constexpr int CLUSTER_ROWS = 72;
+
+// Whether the current device (`device`) can hold a cluster of `blocks` blocks of
+// the solve, asked with the most shared memory that a plan takes and once per
+// device and size: sixteen blocks are beyond the portable size, and a device (or
+// a partition of one) whose GPCs cannot hold them runs k_pcg instead.  Sets the
+// kernel's attributes on the device.
+constexpr int CLUSTER_DEVICES = 64, CLUSTER_SIZES = 5;   // 1, 2, 4, 8, 16
+static bool cluster_fits(int device, int blocks) {
+  static std::mutex mutex;
+  static signed char known[CLUSTER_DEVICES][CLUSTER_SIZES] = {};   // 0 not asked, 1 fits, -1 does not
+  if (device < 0 || device >= CLUSTER_DEVICES) return false;
+  int size = 0;
+  while ((1 << size) < blocks) ++size;
+  std::lock_guard<std::mutex> lock(mutex);
+  signed char& k = known[device][size];
+  if (k == 0) {
+    const void* kernel = (const void*)k_pcg_cluster;
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute at[1];
+    int clusters = 0;
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PCG_SMEM_MAX);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    cluster_config(cfg, at, blocks, CLUSTER_THREADS, PCG_SMEM_MAX, nullptr);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveClusters(&clusters, kernel, &cfg);
+    if (e != cudaSuccess) cudaGetLastError();
+    k = e == cudaSuccess && clusters > 0 ? 1 : -1;
+  }
+  return k > 0;
+}
+
 static bool cluster_plan(const ibl_ctx* c, const PcgArgs& A, ClusterArgs& S, int& blocks, size_t& smem) {
   const int m = c->m_total;
   if (c->sep_on || c->precond_kind != -1 || c->resident_rows != -1 || m > CLUSTER_MARKERS) return false;
@@ -2576,27 +2616,13 @@ static bool cluster_plan(const ibl_ctx* c, const PcgArgs& A, ClusterArgs& S, int
   const size_t g = std::min(up((size_t)S.rows * 64 * (sizeof(df) + sizeof(unsigned short))), PCG_SMEM_MAX - o);
   S.g_bytes = (int)g;
   smem = std::max(o + g, GJ_SMEM);
-  return true;
+  return cluster_fits(c->device, blocks);
 }
 
 static cudaError_t launch_cluster(ibl_ctx* c, PcgArgs& A, ClusterArgs& S, int blocks, size_t smem) {
-  static bool attr_set = false;
-  if (!attr_set) {
-    IBL_CU(cudaFuncSetAttribute((const void*)k_pcg_cluster, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PCG_SMEM_MAX));
-    IBL_CU(cudaFuncSetAttribute((const void*)k_pcg_cluster, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
-    attr_set = true;
-  }
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(blocks);
-  cfg.blockDim = dim3(CLUSTER_THREADS);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = c->stream;
   cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = blocks;
-  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
-  cfg.attrs = at;
-  cfg.numAttrs = 1;
+  cluster_config(cfg, at, blocks, CLUSTER_THREADS, smem, c->stream);
   return cudaLaunchKernelEx(&cfg, k_pcg_cluster, A, S);
 }
 

@@ -77,3 +77,23 @@ def test_marker_list_capacity_without_lists(ibl):
     ok = ibl.from_workload(cfg)
     ok.ibl_step(1)
     ok.ibl_sync()
+
+
+@pytest.mark.parametrize("overlap", [0, 1])
+def test_sixteen_block_cluster(ibl, overlap):
+    """2 x 304 markers, the sixteen-block size, alone and beside the bulk collide."""
+    cfg = _wings(9.0, False)
+    assert sum(len(b["X0"]) for b in cfg["bodies"]) == 608
+    a, b = ibl.from_workload(cfg), ibl.from_workload(cfg)
+    b.ibl_solver_preconditioner(0, -1)
+    sim = oracle_from_workload(cfg)
+    for c in (a, b):
+        c.ibl_set_overlap(overlap)
+        c.ibl_step(8)
+    sim.step(8)
+    compare_fields(a, sim, ibl, TOL_FIELD_FP64)
+    assert rel_err(a.ibl_get_field(ibl.IBL_FIELD_U), b.ibl_get_field(ibl.IBL_FIELD_U)) < TOL_FIELD_FP64
+    again = ibl.from_workload(cfg)
+    again.ibl_set_overlap(1 - overlap)
+    again.ibl_step(8)
+    assert np.array_equal(again.ibl_get_populations(), a.ibl_get_populations())
