@@ -2548,10 +2548,11 @@ cudaError_t ib_step_front(ibl_ctx* c) {
 }
 
 // The solve on one cluster: for marker sets up to CLUSTER_MARKERS, with the
-// automatic preconditioner (an explicit kind or streamed rows keep k_pcg, whose
-// block count the caller may then choose).  One block per CLUSTER_ROWS rows,
-// 1 to 16.
-// G and M stay in shared memory when they fit, else they are read from L2.
+// automatic preconditioner (an explicit kind keeps k_pcg, whose block count the
+// caller may then choose).  One block per CLUSTER_ROWS rows, 1 to 16.  M stays in
+// shared memory (at most 193 KB with everything else) unless the caller asked
+// for rows read from L2, which are multiplied in the same order; G stays there
+// when it fits, else it is read from L2.
 constexpr int CLUSTER_ROWS = 72;
 
 // Whether the current device (`device`) can hold a cluster of `blocks` blocks of
@@ -2585,7 +2586,7 @@ static bool cluster_fits(int device, int blocks) {
 
 static bool cluster_plan(const ibl_ctx* c, const PcgArgs& A, ClusterArgs& S, int& blocks, size_t& smem) {
   const int m = c->m_total;
-  if (c->sep_on || c->precond_kind != -1 || c->resident_rows != -1 || m > CLUSTER_MARKERS) return false;
+  if (c->sep_on || c->precond_kind != -1 || m > CLUSTER_MARKERS) return false;
   blocks = 1;
   while (blocks < CLUSTER_MAX && blocks * CLUSTER_ROWS < m) blocks *= 2;
   const int rows = (m + blocks - 1) / blocks;
@@ -2608,7 +2609,7 @@ static bool cluster_plan(const ibl_ctx* c, const PcgArgs& A, ClusterArgs& S, int
   for (auto& b : c->bodies) slot = std::max(slot, precond_ld(b.m));
   const size_t mrows = sizeof(float) * (size_t)S.rows * slot;
   S.o_m = (int)o;
-  S.slot = o + mrows <= PCG_SMEM_MAX ? slot : 0;
+  S.slot = c->resident_rows != 0 ? slot : 0;
   if (S.slot) o += up(mrows);
   S.o_g = (int)o;
   if (o > PCG_SMEM_MAX) return false;

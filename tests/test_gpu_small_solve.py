@@ -97,3 +97,16 @@ def test_sixteen_block_cluster(ibl, overlap):
     again.ibl_set_overlap(1 - overlap)
     again.ibl_step(8)
     assert np.array_equal(again.ibl_get_populations(), a.ibl_get_populations())
+
+
+@pytest.mark.parametrize("chord", [4.0, 7.9])
+def test_rows_read_from_l2(ibl, chord):
+    """Preconditioner rows kept on chip and read from L2 give the same bits, with the automatic kind too."""
+    cfg = _wings(chord, True)
+    runs = []
+    for resident in (-1, 0):
+        ctx = ibl.from_workload(cfg)
+        ctx.ibl_solver_preconditioner(-1, resident)
+        ctx.ibl_step(10)
+        runs.append(ctx.ibl_get_populations())
+    assert np.array_equal(runs[0], runs[1])
