@@ -570,7 +570,7 @@ ibl_status ibl_step(ibl_ctx* c, int64_t n) {
       CK(cudaEventRecord(c->ev_tiles, c->stream), "event");
       CK(cudaStreamWaitEvent(c->stream_bulk, c->ev_tiles, 0), "stream wait");
       if (ev[4]) CK(cudaEventRecord(ev[4], c->stream_bulk), "event");
-      CK(launch_collide_bulk(c, std::max(1, num_sms() - pcg_block_count(c)), c->stream_bulk), "bulk collide");
+      CK(launch_collide_bulk(c, std::max(1, num_sms() - solve_sms(c)), c->stream_bulk), "bulk collide");
       if (ev[5]) CK(cudaEventRecord(ev[5], c->stream_bulk), "event");
       CK(cudaEventRecord(c->ev_bulk, c->stream_bulk), "event");
       CK(ib_step_back(c), "IB step");

@@ -26,6 +26,7 @@
 //   (end of k_pcg)   F_w = -sum_l 2 rho_l w_l per body in FP64, fixed order.
 #include <cooperative_groups.h>
 
+#include <algorithm>
 #include <cmath>
 #include <mutex>
 
@@ -2402,7 +2403,7 @@ void phase_mark(ibl_ctx* c, int phase) {
 // marker sets too large to split for (the solve then dominates the step);
 // fixed per context so that the solve's reduction order does not depend on
 // the schedule.
-int pcg_block_count(const ibl_ctx* c) {
+static int pcg_block_count(const ibl_ctx* c) {
   const bool half = c->overlap == 1 || c->m_total <= SPLIT_MAX_MARKERS;
   const int want = c->pcg_blocks > 0 ? c->pcg_blocks : (half ? num_sms() / 2 : num_sms());
   return std::max(1, std::min(std::min(std::min(want, num_sms()), MAX_PCG_BLOCKS), c->m_total));
@@ -2584,7 +2585,7 @@ static bool cluster_fits(int device, int blocks) {
   return k > 0;
 }
 
-static bool cluster_plan(const ibl_ctx* c, const PcgArgs& A, ClusterArgs& S, int& blocks, size_t& smem) {
+static bool cluster_plan(const ibl_ctx* c, ClusterArgs& S, int& blocks, size_t& smem) {
   const int m = c->m_total;
   if (c->sep_on || c->precond_kind != -1 || m > CLUSTER_MARKERS) return false;
   blocks = 1;
@@ -2596,9 +2597,9 @@ static bool cluster_plan(const ibl_ctx* c, const PcgArgs& A, ClusterArgs& S, int
   const auto up = [](size_t b) { return (b + 15) & ~(size_t)15; };
   size_t o = up(sizeof(float) * 3 * (size_t)m);
   S.o_xa = (int)o;
-  o = std::max(o + up(sizeof(float) * (size_t)A.vtotal), up(sizeof(df) * 3 * (size_t)m));   // w0 lies on z and A p
+  o = std::max(o + up(sizeof(float) * c->xf_floats), up(sizeof(df) * 3 * (size_t)m));   // w0 lies on z and A p
   S.o_xr = (int)o;
-  o += up(sizeof(float) * (size_t)A.vtotal);
+  o += up(sizeof(float) * c->xf_floats);
   S.o_ys = (int)o;
   o += up(sizeof(float) * 3 * (size_t)S.rows);
   S.o_meta = (int)o;
@@ -2618,6 +2619,23 @@ static bool cluster_plan(const ibl_ctx* c, const PcgArgs& A, ClusterArgs& S, int
   S.g_bytes = (int)g;
   smem = std::max(o + g, GJ_SMEM);
   return cluster_fits(c->device, blocks);
+}
+
+// SMs that a split step's bulk collide leaves to the IB chain.  Beside a cluster
+// these are not the cooperative solve's blocks: a bulk that fills more of the chip
+// leaves no GPC with room for the cluster (each kernel fills an SM's registers)
+// and the solve waits for its end, one that fills less becomes the longer part.
+// us a step with 32, 48, 64 and 76 SMs left, FP32 wings: 520 markers 96^3 150, 140,
+// 141, 141; 128^3 155, 150, 149, 145; 144^3 151, 155, 161, 177; 180^3 218, 226, 269,
+// 272; 608 markers (sixteen blocks) 96^3 159, 143, 138, 138; 160^3 254, 180, 208, 233.
+constexpr long long CLUSTER_FREE_CELLS = 1LL << 21;   // half the SMs up to here, then 48
+constexpr int CLUSTER_FREE_SMS = 48;
+int solve_sms(const ibl_ctx* c) {
+  ClusterArgs S;
+  int blocks = 0;
+  size_t smem = 0;
+  if (!cluster_plan(c, S, blocks, smem)) return pcg_block_count(c);
+  return std::min({c->N > CLUSTER_FREE_CELLS ? CLUSTER_FREE_SMS : num_sms() / 2, num_sms() / 2, c->m_total});
 }
 
 static cudaError_t launch_cluster(ibl_ctx* c, PcgArgs& A, ClusterArgs& S, int blocks, size_t smem) {
@@ -2734,7 +2752,7 @@ cudaError_t ib_step_back(ibl_ctx* c) {
   ClusterArgs S;
   int cluster = 0;
   size_t cluster_smem = 0;
-  if (cluster_plan(c, A, S, cluster, cluster_smem)) {
+  if (cluster_plan(c, S, cluster, cluster_smem)) {
     IBL_CU(launch_cluster(c, A, S, cluster, cluster_smem));
   } else {
     static bool smem_set = false;

@@ -242,14 +242,15 @@ cudaError_t ib_step_front(ibl_ctx* c);    // kinematics and the band tiles of th
 cudaError_t ib_step_back(ibl_ctx* c);     // interpolation .. solve .. spreading
 int num_sms();
 void phase_mark(ibl_ctx* c, int phase);   // ibl_profile level 2 only
-int pcg_block_count(const ibl_ctx* c);
+int solve_sms(const ibl_ctx* c);          // SMs that a split step's bulk collide leaves free
 // Marker count up to which the step is split automatically: beyond it the
 // solve (dense per-body preconditioner, m^2 per iteration) dominates and
 // gets every SM.
 constexpr int SPLIT_MAX_MARKERS = 8192;
 // Cells from which the step is split: 96^3 with 2 x 260 markers takes 137 us a
 // step split and 148 unsplit, 800 x 400 with 2 x 34 markers 105 and 107, 200 x 100
-// 75 and 70.
+// 75 and 70.  With the cooperative solve (FP32 wings): 80^3 with 912 markers 162
+// and 173, 100^3 with 1224 markers 197 and 219, with 1552 224 and 245.
 constexpr long long SPLIT_MIN_CELLS = 1LL << 18;
 cudaError_t launch_force_field(ibl_ctx* c, double* d_out);
 
