@@ -194,11 +194,21 @@ cudaError_t xfer_chunks(const XferSet& s, int t, int threads, cudaStream_t st, c
   return e;
 }
 
+// Whether `host` is pageable memory that CUDA does not know.  Pinned and managed
+// memory is copied directly (a pinned field by one DMA), and a pointer that is
+// not the host's is left to cudaMemcpyAsync's own checks.
+bool pageable(const void* host) {
+  cudaPointerAttributes at;
+  if (cudaPointerGetAttributes(&at, host) == cudaSuccess) return at.type == cudaMemoryTypeUnregistered;
+  cudaGetLastError();
+  return false;
+}
+
 // Copy between device and host memory, ordered on the context's stream; large
-// ones have landed on return, small ones like cudaMemcpyAsync.
+// pageable ones have landed on return, others like cudaMemcpyAsync.
 cudaError_t host_copy(ibl_ctx* c, void* dev, void* host, size_t bytes, bool up) {
   XferSet s;
-  if (bytes < XFER_MIN || !xfer_take(c->device, s))
+  if (bytes < XFER_MIN || !pageable(host) || !xfer_take(c->device, s))
     return up ? cudaMemcpyAsync(dev, host, bytes, cudaMemcpyHostToDevice, c->stream)
               : cudaMemcpyAsync(host, dev, bytes, cudaMemcpyDeviceToHost, c->stream);
   const int threads = std::max(1, std::min({XFER_THREADS, (int)std::thread::hardware_concurrency() / 2,

@@ -161,3 +161,23 @@ def test_init_rounds_as_fp64(ibl, q, shape):
         # f was read as g + w in FP64, which holds all of g above 2^-20
         large = np.abs(g) > 2.0 ** -20
         assert np.array_equal((f[i] - w[i]).astype(np.float32)[large], g.astype(np.float32)[large])
+
+
+def test_pinned_fields_are_copied_directly(ibl):
+    """A velocity field in pinned memory goes up in one copy: the same populations as from pageable memory, and
+    the call's processor time stays near one thread's (staged through the pinned chunks, several threads copy)."""
+    import time
+    torch = pytest.importorskip("torch")
+    shape = (160, 160, 160)
+    pinned = torch.empty((3,) + shape, dtype=torch.float64).pin_memory().numpy()
+    pinned[:] = np.random.default_rng(5).uniform(-0.05, 0.05, size=pinned.shape)
+    ctx = _ctx(ibl, 19, shape, "fp32")
+    ctx.ibl_init_fluid(None, pinned.copy())
+    want = ctx.ibl_get_field(ibl.IBL_FIELD_U)
+    ratios = []
+    for _ in range(6):
+        cpu, wall = time.process_time(), time.perf_counter()
+        ctx.ibl_init_fluid(None, pinned)
+        ratios.append((time.process_time() - cpu) / (time.perf_counter() - wall))
+    assert np.array_equal(ctx.ibl_get_field(ibl.IBL_FIELD_U), want)
+    assert min(ratios) < 1.5
