@@ -121,6 +121,18 @@ std::mutex g_xfer_mutex;
 std::vector<XferSet> g_xfer_free;
 int g_contexts = 0;
 
+// Makes a device current for a scope.
+struct DeviceScope {
+  int before = 0;
+  bool changed = false;
+  explicit DeviceScope(int device) {
+    changed = cudaGetDevice(&before) == cudaSuccess && before != device && cudaSetDevice(device) == cudaSuccess;
+  }
+  ~DeviceScope() {
+    if (changed) cudaSetDevice(before);
+  }
+};
+
 void xfer_free(XferSet& s) {
   if (s.pin) cudaFreeHost(s.pin);
   for (auto& e : s.ev)
@@ -138,6 +150,7 @@ bool xfer_take(int device, XferSet& s) {
         return true;
       }
   }
+  const DeviceScope scope(device);   // the events belong to the device of the streams that they are recorded on
   s.device = device;
   bool ok = cudaMallocHost(&s.pin, 2 * XFER_THREADS * XFER_CHUNK) == cudaSuccess;
   for (auto& e : s.ev) ok = ok && cudaEventCreateWithFlags(&e, cudaEventDisableTiming) == cudaSuccess;
@@ -162,9 +175,10 @@ void xfer_give(XferSet& s) {
 // One thread's chunks, alternating between its two pinned buffers.
 cudaError_t xfer_chunks(const XferSet& s, int t, int threads, cudaStream_t st, char* dev, char* host, size_t bytes,
                         bool up) {
+  const DeviceScope scope(s.device);   // a new thread starts on device 0
   const size_t n = (bytes + XFER_CHUNK - 1) / XFER_CHUNK;
   size_t pending[2] = {0, 0};   // chunk + 1 in flight from or to each buffer
-  cudaError_t e = cudaSetDevice(s.device);
+  cudaError_t e = cudaSuccess;
   auto drain = [&](int k) {
     if (!pending[k]) return;
     const size_t c = pending[k] - 1;
