@@ -118,7 +118,8 @@ struct XferSet {
 };
 
 std::mutex g_xfer_mutex;
-std::vector<XferSet> g_xfer_free;
+XferSet g_xfer_free[XFER_SETS];   // a fixed array: nothing here may throw through the C interface
+int g_xfer_waiting = 0;
 int g_contexts = 0;
 
 // Makes a device current for a scope.
@@ -143,10 +144,10 @@ void xfer_free(XferSet& s) {
 bool xfer_take(int device, XferSet& s) {
   {
     std::lock_guard<std::mutex> lock(g_xfer_mutex);
-    for (size_t i = 0; i < g_xfer_free.size(); ++i)
+    for (int i = 0; i < g_xfer_waiting; ++i)
       if (g_xfer_free[i].device == device) {
         s = g_xfer_free[i];
-        g_xfer_free.erase(g_xfer_free.begin() + i);
+        g_xfer_free[i] = g_xfer_free[--g_xfer_waiting];
         return true;
       }
   }
@@ -164,8 +165,8 @@ bool xfer_take(int device, XferSet& s) {
 void xfer_give(XferSet& s) {
   {
     std::lock_guard<std::mutex> lock(g_xfer_mutex);
-    if (g_contexts > 0 && (int)g_xfer_free.size() < XFER_SETS) {
-      g_xfer_free.push_back(s);
+    if (g_contexts > 0 && g_xfer_waiting < XFER_SETS) {
+      g_xfer_free[g_xfer_waiting++] = s;
       return;
     }
   }
@@ -351,12 +352,14 @@ ibl_status ibl_destroy(ibl_ctx* c) {
   for (auto& ev : c->pev_pool) cudaEventDestroy(ev);
   if (c->h_stage) cudaFreeHost(c->h_stage);
   if (c->stream) cudaStreamDestroy(c->stream);
-  std::vector<XferSet> unused;
+  XferSet unused[XFER_SETS];
+  int n = 0;
   {
     std::lock_guard<std::mutex> lock(g_xfer_mutex);
-    if (--g_contexts == 0) unused.swap(g_xfer_free);
+    if (--g_contexts == 0)
+      while (g_xfer_waiting > 0) unused[n++] = g_xfer_free[--g_xfer_waiting];
   }
-  for (auto& s : unused) xfer_free(s);
+  while (n > 0) xfer_free(unused[--n]);
   delete c;
   return IBL_OK;
 }
