@@ -335,7 +335,7 @@ __device__ __forceinline__ void interpolate_body(int vblock, int m_total, const 
     df wt = df_mul(w[i], w[4 + j]);
     if (g.D == 3) wt = df_mul(wt, w[8 + q]);
     R drho, u[3];
-    node_moments_fast<Q, T, PULL>(src, node[0], node[1], node[2], p, drho, u);
+    node_moments<Q, T, PULL>(src, node[0], node[1], node[2], p, drho, u);
     acc_fma(acc[0], wt, df_from_float(1.f));
     acc_fma(acc[0], wt, to_df(drho));
     for (int c = 0; c < 3; ++c) acc_fma(acc[1 + c], wt, to_df(u[c]));

@@ -147,36 +147,12 @@ __device__ __forceinline__ void moments_of(const R gg[Q], const FluidParams<R>& 
 }
 
 template <int Q, class T, bool PULL>
-__device__ __forceinline__ void node_moments(const T* __restrict__ src, int x, int y, int z, long long cell,
+__device__ __forceinline__ void node_moments(const T* __restrict__ src, int x, int y, int z,
                                              const FluidParams<typename Store<T>::R>& p,
                                              typename Store<T>::R& drho_out, typename Store<T>::R u[3]) {
-  using R = typename Store<T>::R;
-  R gg[Q];
-  gather_q<Q, T, PULL, R>(src, x, y, z, cell, p, gg);
-  moments_of<Q, R>(gg, p, drho_out, u);
-}
-
-// node_moments with the short pull (the same populations, and so the same bits).
-template <int Q, class T, bool PULL>
-__device__ __forceinline__ void node_moments_fast(const T* __restrict__ src, int x, int y, int z,
-                                                  const FluidParams<typename Store<T>::R>& p,
-                                                  typename Store<T>::R& drho_out, typename Store<T>::R u[3]) {
   typename Store<T>::R gg[Q];
   pull_cell<Q, T, PULL>(src, x, y, z, p, gg);
   moments_of<Q, typename Store<T>::R>(gg, p, drho_out, u);
-}
-
-// The same moments as FP64 rho and u*.
-template <int Q, class T, bool PULL>
-__device__ __forceinline__ void node_rho_u(const T* __restrict__ src, int x, int y, int z, long long cell,
-                                           const FluidParams<typename Store<T>::R>& p, double& rho,
-                                           double u[3]) {
-  typename Store<T>::R drho, uu[3];
-  node_moments<Q, T, PULL>(src, x, y, z, cell, p, drho, uu);
-  rho = 1.0 + (double)drho;
-  u[0] = (double)uu[0];
-  u[1] = (double)uu[1];
-  u[2] = (double)uu[2];
 }
 
 // A storage-precision value as a double-float (exact).

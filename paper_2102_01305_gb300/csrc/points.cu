@@ -23,8 +23,9 @@ constexpr double PT_FIX_LIMIT = 9.0e18 / PT_FIX_SCALE;
 constexpr int PT_BAD_STENCIL = 1;
 constexpr int PT_BAD_RANGE = 2;
 
-// Bins and output tiles: 1024 cells, whose spreading sums (24 bytes a cell in
-// 3D) leave room for eight 256-thread blocks on an SM.  A point is visited by
+// Bins and output tiles: 1024 cells, whose spreading sums (33 bytes a cell in 3D
+// with the padding) and candidate list take 38 KB, five 256-thread blocks on an
+// SM.  A point is visited by
 // every tile that its 4-node stencil reaches, 2.2 on average at 16 x 8 x 8.
 constexpr int PT_X = 16, PT_Y = 8, PT_Z = 8;
 constexpr int PT_X2 = 32, PT_Y2 = 32;
@@ -248,7 +249,7 @@ __global__ void __launch_bounds__(256) k_points_interpolate(int m, const int4* _
     const int x = wrap_once(r.x + (k & 3), g.n[0]), y = wrap_once(r.y + ((k >> 2) & 3), g.n[1]);
     const int z = D == 3 ? wrap_once(r.z + (k >> 4), g.n[2]) : 0;
     R drho, u[3];
-    node_moments_fast<Q, T, PULL>(src, x, y, z, p, drho, u);
+    node_moments<Q, T, PULL>(src, x, y, z, p, drho, u);
     sm[e].v[0] = drho;
     sm[e].v[1] = u[0];
     sm[e].v[2] = u[1];
@@ -276,7 +277,7 @@ __global__ void __launch_bounds__(256) k_cell_moments(const T* __restrict__ src,
   if (x >= p.nx || y >= p.ny) return;
   Mom4<R> o;
   R u[3];
-  node_moments_fast<Q, T, PULL>(src, x, y, z, p, o.v[0], u);
+  node_moments<Q, T, PULL>(src, x, y, z, p, o.v[0], u);
   o.v[1] = u[0];
   o.v[2] = u[1];
   o.v[3] = u[2];
