@@ -306,11 +306,12 @@ ibl_status ibl_solver_blocks(ibl_ctx* ctx, int32_t blocks);
  *           at least 4096 markers, else kind 0; up to 640 markers in all the
  *           solve with kind 0 then runs on one thread-block cluster, whose
  *           size follows from the marker count (ibl_solver_blocks has no
- *           effect on it).
+ *           effect on such steps; a device that cannot hold the cluster runs
+ *           the cooperative solve).
  * A change of kind takes effect at the next step and restarts the solver's
  * warm start.  IBL_EINVAL at the next step if kind 1 is asked for bodies
  * that do not qualify.
- * resident_rows (kind 0): -1 (default) each solve block keeps its
+ * resident_rows (kind 0, asked for or automatic): -1 (default) each solve block keeps its
  * preconditioner rows in shared memory when they fit; 0 the rows are always
  * read from L2/HBM (the path every solve takes when they do not fit).  Both
  * paths multiply the same FP32 rows in the same order, so they give bitwise

@@ -5,10 +5,12 @@
 //   k_kinematics     marker positions X and wall velocities U_B (Eqs. 20-23,
 //                    rotational velocity of Sec. 3.3; the per-body motion
 //                    state comes from the host), stencil base nodes and the
-//                    4-point cosine weights (Eq. 14, FP64, stored as FP32 pairs);
+//                    4-point cosine weights (Eq. 14 in 64-bit integers, FP64 runs
+//                    in FP64; stored as FP32 pairs);
 //   k_mark/assign/append
 //                    grid tiles touched by a stencil get a band slot and a
-//                    list of the markers that touch them;
+//                    list of the markers that touch them (up to 4096 markers
+//                    k_ib_front does these and the kinematics in one kernel);
 //   k_interp_assemble
 //                    one launch, two block ranges: rho_l and u*_l (Eq. 17)
 //                    from the populations of the stencil nodes (moments of
@@ -19,7 +21,7 @@
 //                    components at once in double-float arithmetic, an FP32
 //                    dense per-body approximate inverse as preconditioner,
 //                    rebuilt in-kernel (blocked Gauss-Jordan) every few hundred
-//                    steps;
+//                    steps; k_pcg_cluster the same for small marker sets;
 //   (end of k_pcg)   du(x) = sum_l w_l D(x - X_l) (Eq. 15) into 64-bit
 //                    fixed-point band accumulators (order-independent sums);
 //                    the collide kernel forms F = 2 rho du (Eq. 26) from them;

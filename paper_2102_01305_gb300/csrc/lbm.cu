@@ -841,7 +841,8 @@ template <> struct CellSum<float> {
 
 // rho, u = (sum c_i f_i + G/2)/rho and optionally f itself (FP64) of the
 // current post-streaming populations.  U: the velocity is asked for.
-// 64^3 FP32: 68 us for u when every population is converted to FP64.
+// Bound by FP64 divisions and conversions: u of 64^3 FP32 cells 36 us (of 256^3
+// 1636), 68 us when every population is converted to FP64.
 template <int Q, class T, bool PULL, bool U>
 __global__ void __launch_bounds__(256) k_fields(const T* __restrict__ src, FluidParams<typename Store<T>::R> p,
                                                 double* __restrict__ rho_out, double* __restrict__ u_out,
@@ -952,8 +953,8 @@ __device__ __noinline__ double init_fp64(int i, double rho, double u0, double u1
 // at most 2^-45 of its terms); a value whose rounding to FP32 that error could
 // change (about 1 in 1e4), or that is not finite, is formed in FP64 instead, so
 // the stored values are those of FP64 arithmetic.
-// Bound by FP64 conversions of the given field and, in FP32, by HBM: 256^3
-// FP32 413 us, 5189 us when every direction was formed in FP64 by itself.
+// Bound by FP64 conversions of the given field and the FP32 arithmetic: 256^3
+// FP32 744 us, 5189 us when every direction was formed in FP64 by itself.
 template <int Q, class T, bool GIVEN>
 __global__ void __launch_bounds__(256) k_init_eq(T* __restrict__ dst, long long N, const double* __restrict__ rho_in,
                                                  const double* __restrict__ u_in) {
@@ -1022,9 +1023,9 @@ __global__ void k_set_pop(T* __restrict__ dst, long long N, const double* __rest
 // Fixed-order mass: block b sums cells [b*chunk, (b+1)*chunk) in a fixed
 // strided pattern and a fixed tree; the host-side second pass is a fixed loop.
 // A cell's deviations are summed to FP64's accuracy (CellSum), the cells' sums
-// in FP64, and the cells themselves are counted.  Bound by HBM in
-// FP32 (256^3: 268 us; 1280 us with FP64 conversions and additions per
-// direction and 64-bit index divisions).
+// in FP64, and the cells themselves are counted.  256^3 FP32: 315 us, of which
+// the reads take 190, the sums' arithmetic the rest; 1280 us with FP64
+// conversions and additions per direction and 64-bit index divisions.
 template <int Q, class T, bool PULL>
 __global__ void __launch_bounds__(256) k_mass(const T* __restrict__ src, FluidParams<typename Store<T>::R> p,
                                               double* __restrict__ partials, long long chunk) {
