@@ -2581,8 +2581,11 @@ static bool cluster_fits(int device, int blocks) {
     if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     cluster_config(cfg, at, blocks, CLUSTER_THREADS, PCG_SMEM_MAX, nullptr);
     if (e == cudaSuccess) e = cudaOccupancyMaxActiveClusters(&clusters, kernel, &cfg);
-    if (e != cudaSuccess) cudaGetLastError();
-    k = e == cudaSuccess && clusters > 0 ? 1 : -1;
+    if (e != cudaSuccess) {   // not an answer: asked again next time
+      cudaGetLastError();
+      return false;
+    }
+    k = clusters > 0 ? 1 : -1;
   }
   return k > 0;
 }
